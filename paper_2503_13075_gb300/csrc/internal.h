@@ -32,17 +32,12 @@ namespace ilves {
 
 constexpr uint32_t kNoAtom32 = 0xFFFFFFFFu;
 
-// Program words.  IdxT is uint16_t for molecules run by one warp (compact, staged in
-// shared memory) and uint32_t for large molecules run by a whole CTA.
+// Program words of large molecules (32-bit, run by a whole CTA or several); the batched
+// kernel's molecules have a program of their own (BatchLayout).
 //   Task (large molecules): row, col of the target entry; atomsign = (shared atom << 1) |
 //         (sign product < 0), the dummy atom for fill entries, unused for DIAG tasks;
 //         tstart = first term.  Task t's terms are [tstart_t, tstart_{t+1}); a sentinel
 //         task ends the list.
-//   Task word (warp molecules): 32 bits, see TaskWord; no term pointer: in every level
-//         thread r of the molecule's team (kSlotThreads threads) owns tasks t0 + r,
-//         t0 + r + kSlotThreads, ..., and the terms are stored thread by thread (thread
-//         r's terms of level 0, then of level 1, ...), starting at lane_term[r]; a thread
-//         walks its terms with a running offset.
 //   Term: l = slot of Lt[row, m], u = slot of U[m, col], m = the earlier pivot.
 //   Piv:  diag = first slot of the pivot's U row (its L column follows), nup = |N+(pivot)|.
 //   ConA: local atom ids (i, j) of the constraint at position p.
@@ -51,32 +46,53 @@ template <class IdxT> struct Task { IdxT row, col, atomsign, tstart; };
 template <class IdxT> struct ConA { IdxT i, j; };
 template <class IdxT> struct Piv { IdxT diag, nup; };
 
-// Compact task word: row (8) | col (8) << 8 | shared atom (9) << 16 | negative sign
-// product (1) << 25 | number of terms (6) << 26.
-struct TaskWord {
-    static constexpr uint32_t kMaxTerms = 63, kMaxAtom = 511;
+// Words of a batched molecule's program.  Its values are two to a slot: off-diagonal pair k of the
+// factor (U[j,q], L[q,j]), then pivot p at batch_pivot_base + p, then a zero.
+// PairWord: row j (8) | column q (8) << 8 | shared atom (9) << 16 | negative sign product (1) << 25.
+struct PairWord {
+    static constexpr uint32_t kMaxAtom = 511;
     static ILVES_HD uint32_t row(uint32_t w) { return w & 0xFFu; }
     static ILVES_HD uint32_t col(uint32_t w) { return (w >> 8) & 0xFFu; }
     static ILVES_HD uint32_t atom(uint32_t w) { return (w >> 16) & 0x1FFu; }
     static ILVES_HD uint32_t neg(uint32_t w) { return (w >> 25) & 1u; }
-    static ILVES_HD uint32_t nterm(uint32_t w) { return w >> 26; }
-    static ILVES_HD uint32_t make(uint32_t row, uint32_t col, uint32_t atom, uint32_t neg, uint32_t nterm) {
-        return row | (col << 8) | (atom << 16) | (neg << 25) | (nterm << 26);
+    static ILVES_HD uint32_t make(uint32_t row, uint32_t col, uint32_t atomsign) {
+        return row | (col << 8) | ((atomsign >> 1) << 16) | ((atomsign & 1u) << 25);
     }
 };
+// HeadWord of an item that has terms: slot (12) | pivot (1) << 12 | pairs of terms (6) << 13 | its
+// first pair of terms (13) << 19.
+struct HeadWord {
+    static constexpr uint32_t kMaxTerms = 63, kMaxPairs = 8192;
+    static ILVES_HD uint32_t slot(uint32_t h) { return h & 0xFFFu; }
+    static ILVES_HD bool diag(uint32_t h) { return ((h >> 12) & 1u) != 0u; }
+    static ILVES_HD uint32_t pairs(uint32_t h) { return (h >> 13) & 63u; }
+    static ILVES_HD uint32_t first(uint32_t h) { return h >> 19; }
+    static ILVES_HD uint32_t make(uint32_t slot, bool diag, uint32_t pairs, uint32_t first) {
+        return slot | (diag ? 1u << 12 : 0u) | (pairs << 13) | (first << 19);
+    }
+};
+// TermWord of item (j, q) and earlier pivot m: slots of the pairs (m, j) (12) and (m, q) (12) << 12
+// (a pivot's term: the same slot twice) | m (8) << 24.
+struct TermWord {
+    static ILVES_HD uint32_t a(uint32_t t) { return t & 0xFFFu; }
+    static ILVES_HD uint32_t b(uint32_t t) { return (t >> 12) & 0xFFFu; }
+    static ILVES_HD uint32_t m(uint32_t t) { return t >> 24; }
+    static ILVES_HD uint32_t make(uint32_t a, uint32_t b, uint32_t m) { return a | (b << 12) | (m << 24); }
+};
+// Substitution record of a batched molecule's pivot, two words: first pair of its row (12) |
+// entries of the row (8) << 12 | column of the first (8) << 20, columns of the next three (8 each).
+#ifdef __CUDACC__
+struct BackWord {
+    static ILVES_HD uint32_t slot(uint2 w) { return w.x & 0xFFFu; }
+    static ILVES_HD uint32_t n(uint2 w) { return (w.x >> 12) & 0xFFu; }
+    static ILVES_HD uint32_t q(uint2 w, int k) { return k == 0 ? w.x >> 20 : (w.y >> (8 * (k - 1))) & 0xFFu; }
+};
+#endif
+constexpr uint32_t kNoInc = 0x8000u;  // an absent incidence of a batched molecule's atom
 
-// Term words.  Warp-sized molecules (fewer than 256 constraints and 4096 slots) pack a
-// term in 32 bits: l (12) | u (12) << 12 | m (8) << 24.  Large molecules use 4 x 32 bits.
+// Term words of large molecules: 4 x 32 bits.
 struct TermWide { uint32_t l, u, m, pad; };
 template <class IdxT> struct TermOf;
-template <> struct TermOf<uint16_t> {
-    using T = uint32_t;
-    using TaskT = uint32_t;
-    static ILVES_HD uint32_t l(T t) { return t & 0xFFFu; }
-    static ILVES_HD uint32_t u(T t) { return (t >> 12) & 0xFFFu; }
-    static ILVES_HD uint32_t m(T t) { return t >> 24; }
-    static ILVES_HD T make(uint32_t l, uint32_t u, uint32_t m) { return l | (u << 12) | (m << 24); }
-};
 template <> struct TermOf<uint32_t> {
     using T = TermWide;
     using TaskT = Task<uint32_t>;
@@ -85,7 +101,7 @@ template <> struct TermOf<uint32_t> {
     static ILVES_HD uint32_t m(T t) { return t.m; }
     static ILVES_HD T make(uint32_t l, uint32_t u, uint32_t m) { return TermWide{l, u, m, 0u}; }
 };
-constexpr uint32_t kCompactMaxConstraints = 256, kCompactMaxSlots = 4096, kCompactMaxTerms = 65000;
+constexpr uint32_t kCompactMaxConstraints = 256, kCompactMaxSlots = 4096;
 // Threads of the team that solves one molecule of the batched kernel (whole warps; three
 // warps cut the passes of wide levels at no cost in residency, which shared memory
 // limits to about eight molecules per SM), the batched kernel's CTA size bound and its
@@ -109,12 +125,88 @@ constexpr int kDefaultNarrowAtoms = 100;
 
 ILVES_HD uint32_t align16(uint32_t b) { return (b + 15u) & ~15u; }
 
-// `staged` = bytes a warp copies into shared memory (everything but con_gid, which is
-// read from the global copy of the blob); `bytes` = the whole blob.
-// Partitioned molecules add the Schur-contribution tables (see SepInfo, Contrib).
+// Program of a batched molecule (16-byte aligned sections).  `staged` = bytes a team copies
+// into shared memory (everything but con_gid, which is read from the global copy of the
+// blob); `bytes` = the whole blob.
+//   head      BatchHead
+//   con       uint32 x nc            local atoms i | j << 16 of each position
+//   back      uint32 x 2 nc          substitution records (BackWord)
+//   lvl_piv   uint16 x (nlevel + 1)  positions of each level
+//   lvl_hdr   uint16 x (nlevel + 1)  headers of each level (level 0 has none)
+//   inc4      uint16 x 4 na          first four incidences of each atom in ascending position,
+//                                    p << 1 | (atom is the second atom of p), else kNoInc
+//   over_ptr  uint16 x (nover + 1)   incidences past the fourth of atoms [0, nover) (local atoms
+//   over      uint16 x nover_inc     are ordered by decreasing degree)
+//   aslot     uint16 x na            local atom of each atom slot (ascending global order)
+//   pairs     uint32 x npair         PairWord of every off-diagonal pair of A and its fill, pivot
+//                                    by pivot
+//   hdr       uint32 x nhdr          HeadWord of the items that have terms, level by level (in a
+//                                    level by decreasing number of terms)
+//   terms     uint32 x nterm         TermWords, each item's completed to an even number by a term
+//                                    of the zero slot
+struct BatchSizes { int32_t na, nc, npair, nlevel, nhdr, nterm, nover, nover_inc; };
+// wide32, wide16: the first level from which on no level has more than 32, 16 items with terms;
+// wide_piv: the first level from which on no level has more than 32 pivots.
+struct BatchHead { uint16_t wide32, wide16, wide_piv, pad[5]; };
+struct BatchLayout {
+    uint32_t con, back, lvl_piv, lvl_hdr, inc4, over_ptr, over, aslot, pairs, hdr, terms, staged, con_gid, bytes;
+};
+ILVES_HD BatchLayout batch_layout(const BatchSizes& z) {
+    BatchLayout L;
+    uint32_t o = (uint32_t)sizeof(BatchHead);
+    L.con = o;       o = align16(o + 4u * z.nc);
+    L.back = o;      o = align16(o + 8u * z.nc);
+    L.lvl_piv = o;   o = align16(o + 2u * (z.nlevel + 1));
+    L.lvl_hdr = o;   o = align16(o + 2u * (z.nlevel + 1));
+    L.inc4 = o;      o = align16(o + 8u * z.na);
+    L.over_ptr = o;  o = align16(o + (z.nover > 0 ? 2u * (z.nover + 1) : 0u));
+    L.over = o;      o = align16(o + 2u * z.nover_inc);
+    L.aslot = o;     o = align16(o + 2u * z.na);
+    L.pairs = o;     o = align16(o + 4u * z.npair);
+    L.hdr = o;       o = align16(o + 4u * z.nhdr);
+    L.terms = o;     o = align16(o + 4u * z.nterm);
+    L.staged = o;
+    L.con_gid = o;   o = align16(o + 4u * z.nc);
+    L.bytes = o;
+    return L;
+}
+// Slot of pivot 0 among the values of a batched molecule.  Not before 3 na - 2 nc, so that the
+// set-up's staging of x_old (24 na bytes from rf on) ends before the pivots' values, whose
+// second component holds the starting multipliers by then.
+ILVES_HD int32_t batch_pivot_base(int32_t na, int32_t nc, int32_t npair) {
+    const int32_t st = 3 * na - 2 * nc;
+    return npair > st ? npair : st;
+}
+// State of a batched molecule, after its program.  Float64-class values (float64, or
+// float-float pairs of the same size) take 8 bytes; lp_bytes is the factor element size.  Atom
+// arrays x (SoA), w (2 w; the float-float mode: w), wl (4 w; one more atom, of zero weight, for
+// the fill); per constraint rho (SoA; with `disp`, the float-float mode, only its low float
+// parts), s (`disp`: x_unc,i - x_unc,j), d2, lam, the rows rhof (.w = 4 (w_i + w_j)) and rf; c the
+// factor, two values to a slot: pairs, pivots (1 / pivot, solve vector), the zero, and three
+// slots that substitution may read past a row's end.
+struct BatchState { uint32_t x, w, wl, rho, s, d2, lam, rhof, rf, c, bytes; };
+ILVES_HD BatchState batch_state(uint32_t na, uint32_t nc, uint32_t npair, uint32_t lp_bytes, bool disp) {
+    BatchState S;
+    uint32_t o = 0;
+    S.x = o;    o = align16(o + 24u * na);
+    S.w = o;    o = align16(o + 8u * (na + 1));
+    S.wl = o;   o = align16(o + lp_bytes * (na + 1));
+    S.rho = o;  o = align16(o + (disp ? 12u : 24u) * nc);
+    S.s = o;    o = align16(o + (disp ? 24u * nc : 0u));
+    S.d2 = o;   o = align16(o + 8u * nc);
+    S.lam = o;  o = align16(o + 8u * nc);
+    S.rhof = o; o = align16(o + 4u * lp_bytes * nc);
+    S.rf = o;   o = align16(o + 4u * lp_bytes * nc);
+    S.c = o;
+    o = align16(o + 2u * lp_bytes * ((uint32_t)batch_pivot_base((int32_t)na, (int32_t)nc, (int32_t)npair) + nc + 4u));
+    S.bytes = o;
+    return S;
+}
+
+// Program of a large molecule, in global memory.  Partitioned molecules add the Schur-contribution tables (see SepInfo, Contrib).
 struct ProgLayout {
-    uint32_t seg, con_atoms, piv, lvl_task, lvl_piv, lane_term, inc_ptr, inc, atom_off, tasks, terms, sep_info,
-        cptr, cent, pprog_off, pprog, staged, con_gid, bytes;
+    uint32_t seg, con_atoms, piv, lvl_task, lvl_piv, inc_ptr, inc, tasks, terms, sep_info, cptr, cent, pprog_off,
+        pprog, con_gid, bytes;
 };
 
 // Partitioned molecules: the separator block's entries receive the terms of interior
@@ -292,18 +384,15 @@ ILVES_HD ProgLayout prog_layout(uint32_t na, uint32_t nc, uint32_t ntask, uint32
                                 uint32_t pprog_bytes = 0) {
     ProgLayout L;
     const uint32_t ix = (uint32_t)sizeof(IdxT);
-    const bool compact = ix == 2u;
     uint32_t o = 0;
     L.seg = o;       o = align16(o + 12u * (n_seg + 1));
     L.con_atoms = o; o = align16(o + 2u * ix * nc);
     L.piv = o;       o = align16(o + 2u * ix * nc);
     L.lvl_task = o;  o = align16(o + ix * (nlevel + 1));
     L.lvl_piv = o;   o = align16(o + ix * (nlevel + 1));
-    L.lane_term = o; o = align16(o + (compact ? ix * (uint32_t)kSlotThreads : 0u));
     L.inc_ptr = o;   o = align16(o + ix * (na + 1));
     L.inc = o;       o = align16(o + ix * 2u * nc);
-    L.atom_off = o;  o = align16(o + (compact ? ix * na : 0u));  // atom slot -> local atom
-    L.tasks = o;     o = align16(o + (compact ? 4u * ntask : 4u * ix * (ntask + 1)));
+    L.tasks = o;     o = align16(o + 4u * ix * (ntask + 1));
     L.terms = o;     o = align16(o + (uint32_t)sizeof(typename TermOf<IdxT>::T) * nterm);
     const bool parted = n_seg > 1;
     L.sep_info = o;  o = align16(o + (parted ? 8u * n_sept : 0u));
@@ -311,7 +400,6 @@ ILVES_HD ProgLayout prog_layout(uint32_t na, uint32_t nc, uint32_t ntask, uint32
     L.cent = o;      o = align16(o + (parted ? 16u * n_cent : 0u));
     L.pprog_off = o; o = align16(o + (pprog_bytes ? 4u * (n_seg + 1) : 0u));  // parts, separators, end
     L.pprog = o;     o = align16(o + pprog_bytes);
-    L.staged = o;
     L.con_gid = o;   o = align16(o + 4u * nc);
     L.bytes = o;
     return L;
@@ -354,7 +442,7 @@ ILVES_HD StateLayout state_layout(uint32_t na, uint32_t nc, uint32_t ntask, uint
     return S;
 }
 
-// One molecule as the kernels see it (72 bytes).
+// One molecule as the kernels see it.
 struct MolDesc {
     int64_t blob_off;    // byte offset of the program blob in the blob buffer (16-B aligned)
     int64_t work_off;    // large path: byte offset of the numerical state in the workspace
@@ -370,6 +458,10 @@ struct MolDesc {
     int32_t n_cent;  // partitioned: Schur contribution entries over all parts
     int32_t pprog_bytes;  // partitioned: bytes of the segment programs (parts, then separators)
     int32_t opm;          // overlapping domains: overlap depth (0 = not solved by domains)
+    int32_t n_hdr, n_over, n_over_inc, n_pair;  // batched: see BatchSizes (nterm: the completed terms)
 };
+ILVES_HD BatchSizes batch_sizes(const MolDesc& D) {
+    return BatchSizes{D.na, D.nc, D.n_pair, D.nlevel, D.n_hdr, D.nterm, D.n_over, D.n_over_inc};
+}
 
 }  // namespace ilves

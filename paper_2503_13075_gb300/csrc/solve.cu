@@ -72,14 +72,61 @@ __device__ __forceinline__ bool abs_le(double s, double t) {
     const long long sb = __double_as_longlong(s) & 0x7FFFFFFFFFFFFFFFll;
     return sb <= __double_as_longlong(t);
 }
+// |s| <= tol * d2, settled in float32 unless the two are within 2^-20 of each other (or out of
+// the middle of float32's range): the float64 product would cost a pipe slot of 66 cycles.
+// narrow() truncates, so both float32 values are at most 2^-21 off.
+__device__ __forceinline__ bool within(double s, double tol, double d2) {
+    const float sf = fabsf(narrow(s)), tf = narrow(tol) * narrow(d2);
+    if (tf > 1e-30f && tf < 1e30f) {
+        if (sf > tf * (1.0f + 0x1p-20f)) return false;
+        if (sf < tf * (1.0f - 0x1p-20f)) return true;
+    }
+    return abs_le(s, tol * d2);
+}
 __device__ __forceinline__ bool nonfinite(double s) {
     return (__double_as_longlong(s) & 0x7FF0000000000000ll) == 0x7FF0000000000000ll;
 }
 __device__ __forceinline__ bool nonfinite(float s) { return (__float_as_uint(s) & 0x7F800000u) == 0x7F800000u; }
 __device__ __forceinline__ float lp_abs(float v) { return fabsf(v); }
 __device__ __forceinline__ double lp_abs(double v) { return fabs(v); }
-__device__ __forceinline__ float lp_rcp(float a) { return __frcp_rn(a); }
-__device__ __forceinline__ double lp_rcp(double a) { return 1.0 / a; }
+// Reciprocal of a pivot.  float32: the hardware approximation and one Newton step by fused
+// multiply-adds (Markstein's theorem), the correctly rounded value for every normal a with a
+// normal 1 / a (compared with __frcp_rn over all 2^32 inputs); about 35 cycles where the
+// general routine takes 93.
+__device__ __forceinline__ float lp_rcp(float a) {
+    const unsigned e = (__float_as_uint(a) >> 23) & 0xFFu;
+    if (e - 1u >= 252u) return __frcp_rn(a);  // zero, subnormal, infinite, NaN, or a subnormal result
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return __fmaf_rn(r, __fmaf_rn(-a, r, 1.0f), r);
+}
+// float64: a float32 seed (relative error below 2^-21) and one cubic Newton step,
+// r (1 + e + e^2) with e = 1 - a r: three float64 instructions, where the division takes
+// about six (a warp's float64 instruction holds its scheduler's pipe for 66 cycles on this GPU:
+// 230 against 368 cycles).  The truncated terms are below 2^-63, so only the last FMA rounds.
+__device__ __forceinline__ double lp_rcp(double a) {
+    const int e = (__double2hiint(a) >> 20) & 0x7FF;
+    if (e < 1023 - 120 || e > 1023 + 120) return 1.0 / a;
+    float s;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(narrow(a)));
+    const double r = widen(s);
+    const double d = fma(-a, r, 1.0);
+    return fma(r, fma(d, d, d), r);
+}
+// A pivot s vanished against its assembled entry a: !(|s| > pivot_rel |a|).  float64: settled
+// on the exponents alone unless |s| is below about 2^-42 |a|, since a comparison and a product
+// in float64 cost two pipe slots of 66 cycles.
+template <class Mode>
+__device__ __forceinline__ bool pivot_vanished(float s, float a) {
+    return !(lp_abs(s) > Mode::pivot_rel * lp_abs(a));
+}
+template <class Mode>
+__device__ __forceinline__ bool pivot_vanished(double s, double a) {
+    static_assert(Mode::pivot_rel < 0x1p-43, "the exponent test below");
+    const int es = (__double2hiint(s) >> 20) & 0x7FF, ea = (__double2hiint(a) >> 20) & 0x7FF;
+    if (es >= ea - 42 && es < 0x7FF && ea < 0x7FF && es > 0) return false;
+    return !(lp_abs(s) > Mode::pivot_rel * lp_abs(a));
+}
 
 // ------------------------------------------------------------------------------------
 // float-float arithmetic: a value is the unevaluated sum hi + lo of two float32 words
@@ -162,6 +209,7 @@ __device__ __forceinline__ double as_bits(dfloat v) { return *reinterpret_cast<d
 template <int kThreads>
 struct SlotTeamT {
     static constexpr int kSize = kThreads;
+    static constexpr bool kWarp = kThreads == 32;
     __device__ __forceinline__ int rank() const { return threadIdx.x % kThreads; }
     __device__ __forceinline__ int size() const { return kThreads; }
     __device__ __forceinline__ int id() const { return threadIdx.x / kThreads; }
@@ -198,8 +246,6 @@ struct SlotTeamT {
 };
 using SlotTeam = SlotTeamT<kSlotThreads>;
 using NarrowTeam = SlotTeamT<kNarrowThreads>;
-template <class T> struct IsSlotTeam : std::false_type {};
-template <int N> struct IsSlotTeam<SlotTeamT<N>> : std::true_type {};
 struct BlockTeam {
     __device__ __forceinline__ int rank() const { return threadIdx.x; }
     __device__ __forceinline__ int size() const { return blockDim.x; }
@@ -319,7 +365,6 @@ struct MolView {
     using TO = TermOf<IdxT>;
     using TaskT = typename TO::TaskT;
     static constexpr bool DF = Mode::df;
-    static constexpr bool kCompact = sizeof(IdxT) == 2;
     int na, nc;
     const SegRow* seg;
     const ConA<IdxT>* con;
@@ -327,10 +372,8 @@ struct MolView {
     const Piv<IdxT>* piv;
     const IdxT* lvl_task;
     const IdxT* lvl_piv;
-    const IdxT* lane_term;
     const IdxT* inc_ptr;
     const IdxT* inc;
-    const IdxT* aslot;  // batched molecules: local atom of each atom slot
     const TaskT* tasks;
     const typename TO::T* terms;
     double *X, *W, *RHO, *SK, *D2, *LAM;
@@ -346,7 +389,6 @@ struct MolView {
     int sep_t0;
     int sep_p0;    // first separator position (nc if not partitioned)
     bool cohall;   // every state load is foreign (the separator phase)
-    double* STG;  // x_old gathered AoS (warp path set-up only; aliases RF and later arrays)
     const MolDesc* D;
     const SolveArgs* A;
     float tolf;  // tol in float (float-float convergence test)
@@ -369,10 +411,8 @@ struct MolView {
         piv = reinterpret_cast<const Piv<IdxT>*>(prog + PL.piv);
         lvl_task = reinterpret_cast<const IdxT*>(prog + PL.lvl_task);
         lvl_piv = reinterpret_cast<const IdxT*>(prog + PL.lvl_piv);
-        lane_term = reinterpret_cast<const IdxT*>(prog + PL.lane_term);
         inc_ptr = reinterpret_cast<const IdxT*>(prog + PL.inc_ptr);
         inc = reinterpret_cast<const IdxT*>(prog + PL.inc);
-        aslot = reinterpret_cast<const IdxT*>(prog + PL.atom_off);
         tasks = reinterpret_cast<const TaskT*>(prog + PL.tasks);
         terms = reinterpret_cast<const typename TO::T*>(prog + PL.terms);
         X = reinterpret_cast<double*>(st + SL.x);
@@ -387,7 +427,6 @@ struct MolView {
         RF = reinterpret_cast<V4*>(st + SL.rf);
         Y = reinterpret_cast<LP*>(st + SL.y);
         V = reinterpret_cast<LP*>(st + SL.vals);
-        STG = reinterpret_cast<double*>(st + SL.stage);
         sep_info = reinterpret_cast<const SepInfo*>(prog + PL.sep_info);
         cptr = reinterpret_cast<const int32_t*>(prog + PL.cptr);
         cent = reinterpret_cast<const Contrib*>(prog + PL.cent);
@@ -396,15 +435,9 @@ struct MolView {
         sep_p0 = d.n_seg > 1 ? ldp<kCoh>(&seg[d.n_seg - 1].piv) : nc;
         cohall = false;
     }
-    // global atom of atom slot o (the molecule's atoms in ascending global order); in
-    //      large molecules local atom a sits in slot a, in batched molecules in the slot
-    //      whose entry of aslot is a (their local atoms are ordered by degree)
-    __device__ __forceinline__ int64_t slot_gid(int o) const {
-        return D->atom_base >= 0 ? (int64_t)D->atom_base + o : (int64_t)A->atom_gid[D->gid_off + o];
-    }
+    // global atom of local atom a (the molecule's atoms in ascending global order)
     __device__ __forceinline__ int64_t gid(int a) const {
-        static_assert(!kCompact, "batched molecules address their atoms by slot");
-        return slot_gid(a);
+        return D->atom_base >= 0 ? (int64_t)D->atom_base + a : (int64_t)A->atom_gid[D->gid_off + a];
     }
     __device__ __forceinline__ ConA<IdxT> cons(int p) const { return ldp<kCoh>(con + p); }
     __device__ __forceinline__ int32_t gid_of_con(int p) const { return __ldg(con_gid + p); }
@@ -548,7 +581,7 @@ struct MolView {
             VS[t] = sacc;
             if (wt) V[T0 + t] = sacc;
             if (diag) {  // rc is a part position
-                singular = singular || !(lp_abs(sacc) > Mode::pivot_rel * lp_abs(a));
+                singular = singular || pivot_vanished<Mode>(sacc, a);
                 const LP ri = lp_rcp(sacc);
                 reinterpret_cast<LP*>(RFS + rc)[3] = ri;
                 const LP ny = YS[rc] - yv;
@@ -708,72 +741,6 @@ struct MolView {
         }
     }
 
-    // ---- S1, shared-memory state: one batch of asynchronous gathers, then local passes.
-    // x_old -> STG (AoS); x_unc -> X (SoA; AoS in the float-float mode, where X is free
-    // until the displacements start); inv_mass -> W, d -> D2, lambda0 -> Y as raw values.
-    //      The reads run over atom slots, so consecutive lanes read consecutive addresses.
-    __device__ __forceinline__ void s1_gather(int r0, int ts) {
-        for (int e = r0; e < 3 * na; e += ts) {
-            const int o = e / 3, c = e - 3 * o, a = (int)aslot[o];
-            const int64_t g = 3 * slot_gid(o) + c;
-            cp_async8(STG + 3 * a + c, A->x_old + g);
-            cp_async8(DF ? X + 3 * a + c : X + c * na + a, A->x_unc + g);
-        }
-        for (int o = r0; o < na; o += ts) cp_async8(W + aslot[o], A->inv_mass + slot_gid(o));
-        for (int p = r0; p < nc; p += ts) {
-            const int32_t g = gid_of_con(p);
-            cp_async8(D2 + p, A->d + g);
-            if (A->lambda0 && !A->start_diag) cp_async4(reinterpret_cast<float*>(Y + p), A->lambda0 + g);
-        }
-        cp_async_wait_all();
-    }
-    __device__ __forceinline__ void s1_atom_local(int a) {
-        const double w = *(W + a);
-        if constexpr (DF) W[a] = as_bits(df_split(w));
-        WL[a] = to_lp<LP>(w);
-    }
-    __device__ __forceinline__ void s1_constraint_local(int p) {
-        const ConA<IdxT> c = cons(p);
-        const int i = c.i, j = c.j;
-        const double rx = *(STG + 3 * i) - *(STG + 3 * j);
-        const double ry = *(STG + 3 * i + 1) - *(STG + 3 * j + 1);
-        const double rz = *(STG + 3 * i + 2) - *(STG + 3 * j + 2);
-        V4 v;
-        v.x = to_lp<LP>(rx);
-        v.y = to_lp<LP>(ry);
-        v.z = to_lp<LP>(rz);
-        v.w = *(WL + i) + *(WL + j);
-        RHOF[p] = v;
-        const double dd = *(D2 + p);
-        if constexpr (DF) {
-            RHOL[p] = df_split(rx).lo;
-            RHOL[nc + p] = df_split(ry).lo;
-            RHOL[2 * nc + p] = df_split(rz).lo;
-            D2[p] = as_bits(df_split(dd * dd));
-            SK[p] = as_bits(df_split(*(X + 3 * i) - *(X + 3 * j)));
-            SK[nc + p] = as_bits(df_split(*(X + 3 * i + 1) - *(X + 3 * j + 1)));
-            SK[2 * nc + p] = as_bits(df_split(*(X + 3 * i + 2) - *(X + 3 * j + 2)));
-        } else {
-            RHO[p] = rx;
-            RHO[nc + p] = ry;
-            RHO[2 * nc + p] = rz;
-            D2[p] = dd * dd;
-        }
-        float l0 = A->lambda0 ? *(reinterpret_cast<const float*>(Y + p)) : 0.0f;
-        if (A->start_diag) {  // x_unc is in X (AoS in the float-float mode, else SoA)
-            float u[3];
-            for (int c = 0; c < 3; ++c)
-                u[c] = DF ? narrow(*(X + 3 * i + c)) - narrow(*(X + 3 * j + c))
-                          : narrow(*(X + c * na + i)) - narrow(*(X + c * na + j));
-            l0 = diag_start(u[0], u[1], u[2], narrow(*(STG + 3 * i)) - narrow(*(STG + 3 * j)),
-                            narrow(*(STG + 3 * i + 1)) - narrow(*(STG + 3 * j + 1)),
-                            narrow(*(STG + 3 * i + 2)) - narrow(*(STG + 3 * j + 2)), narrow(dd),
-                            f32_of(*(WL + i)) + f32_of(*(WL + j)));
-        }
-        LAM[p] = DF ? as_bits(dfloat{l0, 0.0f}) : widen(l0);
-        Y[p] = (LP)l0;
-    }
-
     // ---- S6: x_a -= w_a sum_k s_k(a) 2 Y_k rho_k   (Y holds delta, or lambda0).
     //      upd_eval computes the new coordinates (float64 class, as bit patterns),
     //      upd_store writes them.
@@ -861,7 +828,7 @@ struct MolView {
             const double rz = x_ld(2, i, fx) - x_ld(2, j, fx);
             const double d2 = *(D2 + p);
             const double sg = fma(rx, rx, fma(ry, ry, fma(rz, rz, -d2)));
-            o.conv = abs_le(sg, A->tol * d2);
+            o.conv = within(sg, A->tol, d2);
             o.bad = nonfinite(sg);
             o.v.x = to_lp<LP>(rx);
             o.v.y = to_lp<LP>(ry);
@@ -910,7 +877,7 @@ struct MolView {
         }
         v_st(t, sacc);
         if (diag) {
-            singular = singular || !(lp_abs(sacc) > Mode::pivot_rel * lp_abs(a));
+            singular = singular || pivot_vanished<Mode>(sacc, a);
             inv_st(row, lp_rcp(sacc));
             y_st(row, y_ld(row) - yv);
         }
@@ -921,21 +888,6 @@ struct MolView {
         const int e1 = ldp<kCoh>(tasks + t + 1).tstart;
         task_core(t, tk.row, tk.col, tk.atomsign >> 1, tk.atomsign & 1, tk.tstart, e1, diag, singular);
     }
-    // batched molecules: one level's tasks t0 + lane + kTeam k for a team of kTeam threads
-    //      (the width the program was laid out for); the lane walks its terms from offset e
-    template <int kTeam>
-    __device__ __forceinline__ void level_tasks(int t0, int t1, int np, int lane, int& e, bool& singular) {
-        for (int t = t0 + lane; t < t1; t += kTeam) {
-            const uint32_t w = lds<kCoh>(tasks + t);
-            const int n = (int)TaskWord::nterm(w);
-            const bool diag = t < t0 + np;
-            finish(t, TaskWord::row(w),
-                   assemble(TaskWord::row(w), TaskWord::col(w), TaskWord::atom(w), TaskWord::neg(w), diag), e, e + n,
-                   diag, singular);
-            e += n;
-        }
-    }
-
     // ---- forward S5 alone (ILVES-F iterations after the first): y_p -= sum_m L[p,m] y_m,
     //      with the terms [e0, e1) of pivot p's DIAG task
     __device__ __forceinline__ void forward_terms(int p, int e0, int e1) {
@@ -955,10 +907,7 @@ struct MolView {
     __device__ __forceinline__ void chord_rows(int p) { rf_st(p, *(RHOF + p)); }
 
     // ---- backward S5 for pivot p: delta_p = inv_p (y_p - sum_q U[p,q] delta_q)
-    __device__ __forceinline__ int task_col(int t) const {
-        if constexpr (kCompact) return (int)TaskWord::col(ldp<kCoh>(tasks + t));
-        else return (int)ldp<kCoh>(tasks + t).col;
-    }
+    __device__ __forceinline__ int task_col(int t) const { return (int)ldp<kCoh>(tasks + t).col; }
     __device__ __forceinline__ void backward(int p) {
         const Piv<IdxT> pv = ldp<kCoh>(piv + p);
         const int us = pv.diag, nu = pv.nup;
@@ -1010,7 +959,7 @@ struct MolView {
         }
         V[t] = sacc;
         if (diag) {
-            singular = singular || !(lp_abs(sacc) > Mode::pivot_rel * lp_abs(a));
+            singular = singular || pivot_vanished<Mode>(sacc, a);
             *inv_ptr(tk.row) = lp_rcp(sacc);
             Y[tk.row] = lds<kCoh>(Y + tk.row) - yv;
         }
@@ -1083,7 +1032,7 @@ struct MolView {
         }
         SV[tl] = sacc;
         if (diag) {
-            singular = singular || !(lp_abs(sacc) > Mode::pivot_rel * lp_abs(a));
+            singular = singular || pivot_vanished<Mode>(sacc, a);
             reinterpret_cast<LP*>(SRF + row)[3] = lp_rcp(sacc);
             SY[row] -= yv;
         }
@@ -1124,7 +1073,7 @@ struct MolView {
                 const LP sacc = a + SV[tl] - ps;
                 SV[tl] = sacc;
                 if (diag) {
-                    singular = singular || !(lp_abs(sacc) > Mode::pivot_rel * lp_abs(a));
+                    singular = singular || pivot_vanished<Mode>(sacc, a);
                     reinterpret_cast<LP*>(SRF + row)[3] = lp_rcp(sacc);
                     SY[row] -= py;
                 }
@@ -1192,15 +1141,6 @@ struct MolView {
             A->x_out[3 * g + 2] = *(X + 2 * na + a);
         }
     }
-    // batched molecules: the positions, one coordinate per lane in global order
-    __device__ __forceinline__ void out_atoms_by_slot(int r0, int ts) {
-        for (int e = r0; e < 3 * na; e += ts) {
-            const int o = e / 3, c = e - 3 * o, a = (int)aslot[o];
-            const int64_t g = 3 * slot_gid(o) + c;
-            if constexpr (DF) A->x_out[g] = A->x_unc[g] + df_join(as_df(*(X + c * na + a)));
-            else A->x_out[g] = *(X + c * na + a);
-        }
-    }
     __device__ __forceinline__ void out_lambda(int p) {
         const double l = *(LAM + p);
         A->lambda_out[gid_of_con(p)] = DF ? df_join(as_df(l)) : l;
@@ -1208,39 +1148,23 @@ struct MolView {
 };
 
 // ------------------------------------------------------------------------------------
-// one molecule, one team (a warp with state in shared memory, or a CTA with state in a
-// global workspace)
+// one molecule, one CTA with its state in a global workspace
 // ------------------------------------------------------------------------------------
-template <class Mode, class IdxT, class Team>
-__device__ void solve_molecule(const Team& tm, const MolDesc& D, const uint8_t* prog, uint8_t* st,
-                               const SolveArgs& A, const uint8_t* gprog) {
-    constexpr bool kCompact = sizeof(IdxT) == 2;  // batched-kernel molecules (a SlotTeamT)
-    MolView<Mode, IdxT, false> M;
-    M.init(D, prog, st, A, gprog);
+template <class Mode>
+__device__ void solve_molecule(const BlockTeam& tm, const MolDesc& D, const uint8_t* prog, uint8_t* st,
+                               const SolveArgs& A) {
+    MolView<Mode, uint32_t, false> M;
+    M.init(D, prog, st, A, prog);
     const int na = D.na, nc = D.nc;
     const int r0 = tm.rank(), ts = tm.size();
     // ---- S1
-    if constexpr (IsSlotTeam<Team>::value) {
-        M.s1_gather(r0, ts);
-        tm.sync();
-        for (int a = r0; a < na; a += ts) M.s1_atom_local(a);
-        if (r0 == 0) M.s1_dummy();
-        tm.sync();
-        for (int p = r0; p < nc; p += ts) M.s1_constraint_local(p);
-        tm.sync();
-        if constexpr (Mode::df) {
-            for (int a = r0; a < na; a += ts) M.s1_atom_unc(a);
-            tm.sync();
-        }
-    } else {
-        for (int a = r0; a < na; a += ts) M.s1_atom(a, true);
-        if (r0 == 0) M.s1_dummy();
-        tm.sync();
-        for (int p = r0; p < nc; p += ts) M.s1_constraint(p, true);
-        tm.sync();
-        for (int a = r0; a < na; a += ts) M.s1_atom_unc(a);
-        tm.sync();
-    }
+    for (int a = r0; a < na; a += ts) M.s1_atom(a, true);
+    if (r0 == 0) M.s1_dummy();
+    tm.sync();
+    for (int p = r0; p < nc; p += ts) M.s1_constraint(p, true);
+    tm.sync();
+    for (int a = r0; a < na; a += ts) M.s1_atom_unc(a);
+    tm.sync();
     if (A.has_start()) {  // x = x_unc - M^-1 G(x_old)^T lambda0
         for (int a = r0; a < na; a += ts) M.update_atom(a);
         tm.sync();
@@ -1266,18 +1190,12 @@ __device__ void solve_molecule(const Team& tm, const MolDesc& D, const uint8_t* 
                 for (int p = r0; p < nc; p += ts) M.chord_rows(p);
                 tm.sync();
             }
-            // one pass per level; the first np tasks of a level are its DIAG tasks; a warp
-            // lane walks its terms with a running offset
+            // one pass per level; the first np tasks of a level are its DIAG tasks
             bool singular = false;
-            int e = kCompact ? (int)M.lane_term[r0] : 0;
             for (int l = 0; l < D.nlevel; ++l) {
                 const int p0 = M.lvl_piv[l], np = M.lvl_piv[l + 1] - p0;
                 const int t0 = M.lvl_task[l], t1 = M.lvl_task[l + 1];
-                if constexpr (kCompact) {
-                    M.template level_tasks<Team::kSize>(t0, t1, np, r0, e, singular);
-                } else {
-                    for (int t = t0 + r0; t < t1; t += ts) M.task(t, t < t0 + np, singular);
-                }
+                for (int t = t0 + r0; t < t1; t += ts) M.task(t, t < t0 + np, singular);
                 tm.sync();
             }
             if (tm.any(singular)) {
@@ -1286,19 +1204,9 @@ __device__ void solve_molecule(const Team& tm, const MolDesc& D, const uint8_t* 
                 break;
             }
         } else {  // ILVES-F: forward substitution with the stored factor
-            int e = kCompact ? (int)M.lane_term[r0] : 0;
             for (int l = 0; l < D.nlevel; ++l) {
                 const int p0 = M.lvl_piv[l], p1 = M.lvl_piv[l + 1], t0 = M.lvl_task[l];
-                if constexpr (kCompact) {  // DIAG tasks: t0 + (p - p0); skip the others' terms
-                    const int t1 = M.lvl_task[l + 1];
-                    for (int t = t0 + r0; t < t1; t += ts) {
-                        const int n = (int)TaskWord::nterm(M.tasks[t]);
-                        if (t < t0 + (p1 - p0)) M.forward_terms(p0 + (t - t0), e, e + n);
-                        e += n;
-                    }
-                } else {
-                    for (int p = p0 + r0; p < p1; p += ts) M.forward(t0 + (p - p0), p);
-                }
+                for (int p = p0 + r0; p < p1; p += ts) M.forward(t0 + (p - p0), p);
                 tm.sync();
             }
         }
@@ -1311,9 +1219,7 @@ __device__ void solve_molecule(const Team& tm, const MolDesc& D, const uint8_t* 
         for (int a = r0; a < na; a += ts) M.update_atom(a);
         tm.sync();
     }
-    if constexpr (kCompact) M.out_atoms_by_slot(r0, ts);
-    else
-        for (int a = r0; a < na; a += ts) M.out_atom(a);
+    for (int a = r0; a < na; a += ts) M.out_atom(a);
     if (A.lambda_out)
         for (int p = r0; p < nc; p += ts) M.out_lambda(p);
     if (r0 == 0) {
@@ -1955,7 +1861,7 @@ k_solve_opm(const MolDesc* __restrict__ desc, const uint8_t* __restrict__ blob, 
                 const double d2 = D2[p];
                 const double sg = fma(rx, rx, fma(ry, ry, fma(rz, rz, -d2)));
                 if (CML[p] >> 31) {
-                    conv = conv && abs_le(sg, A.tol * d2);
+                    conv = conv && within(sg, A.tol, d2);
                     bad = bad || nonfinite(sg);
                 }
                 Y[p] = to_lp<LP>(sg);
@@ -2014,7 +1920,7 @@ k_solve_opm(const MolDesc* __restrict__ desc, const uint8_t* __restrict__ blob, 
                 e += n;
                 V[t] = sacc;
                 if (diag) {
-                    singular = singular || !(lp_abs(sacc) > Mode::pivot_rel * lp_abs(a));
+                    singular = singular || pivot_vanished<Mode>(sacc, a);
                     reinterpret_cast<LP*>(RF + rc)[3] = lp_rcp(sacc);
                     Y[rc] -= yv;
                 }
@@ -2089,6 +1995,10 @@ k_solve_opm(const MolDesc* __restrict__ desc, const uint8_t* __restrict__ blob, 
     }
 }
 
+}  // namespace ilves
+#include "batched.cuh"
+namespace ilves {
+
 // ------------------------------------------------------------------------------------
 // kernels
 // ------------------------------------------------------------------------------------
@@ -2144,14 +2054,14 @@ __device__ __forceinline__ void run_slot(const MolDesc* __restrict__ desc, const
     int mol = q < q1 ? S.slot_mol[q] : (P.n > 0 ? pool_ticket(P, tm, box) : -1);
     while (mol >= 0) {
         const MolDesc D = desc[mol];
-        const ProgLayout PL = prog_layout<uint16_t>(D.na, D.nc, D.ntask, D.nterm, D.nlevel, D.n_seg);
+        const BatchLayout PL = batch_layout(batch_sizes(D));
         const uint4* src = reinterpret_cast<const uint4*>(blob + D.blob_off);
         uint4* dst = reinterpret_cast<uint4*>(slice);
         const int n16 = (int)(PL.staged >> 4);
         for (int k = lane; k < n16; k += Team::kSize) cp_async16(dst + k, src + k);  // all in flight
         if (q + 1 < q1) {  // the next queued molecule's program and atom inputs into L2 meanwhile
             const MolDesc Dn = desc[S.slot_mol[q + 1]];
-            const uint32_t nb = prog_layout<uint16_t>(Dn.na, Dn.nc, Dn.ntask, Dn.nterm, Dn.nlevel, Dn.n_seg).bytes;
+            const uint32_t nb = batch_layout(batch_sizes(Dn)).bytes;
             const uint8_t* pb = blob + Dn.blob_off;
             constexpr uint32_t kStep = 128u * Team::kSize;
             for (uint32_t o = 128u * lane; o < nb; o += kStep) prefetch_l2(pb + o);
@@ -2168,7 +2078,7 @@ __device__ __forceinline__ void run_slot(const MolDesc* __restrict__ desc, const
         }
         cp_async_wait_all();
         tm.sync();
-        solve_molecule<Mode, uint16_t, Team>(tm, D, slice, slice + PL.staged, A, blob + D.blob_off);
+        solve_batched<Mode, Team>(tm, D, PL, slice, A, blob + D.blob_off);
         tm.sync();
         ++q;
         mol = q < q1 ? S.slot_mol[q] : (P.n > 0 ? pool_ticket(P, tm, box) : -1);
@@ -2215,7 +2125,7 @@ k_solve_large(const MolDesc* __restrict__ desc, const uint8_t* __restrict__ blob
               SolveArgs A) {
     const BlockTeam tm;
     const MolDesc D = desc[blockIdx.x];
-    solve_molecule<Mode, uint32_t, BlockTeam>(tm, D, blob + D.blob_off, work + D.work_off, A, blob + D.blob_off);
+    solve_molecule<Mode>(tm, D, blob + D.blob_off, work + D.work_off, A);
 }
 
 __global__ void k_copy_free(const int32_t* __restrict__ idx, int n, const double* __restrict__ x_unc,
@@ -2365,7 +2275,11 @@ static ilves_status upload_topology(ilves_topology* T, const ilves_setup_opts& o
         D.gid_off = (int32_t)gids.size();
         gids.insert(gids.end(), M.atoms.begin(), M.atoms.end());
         D.mol_id = m;
-        D.nterm = M.nterm;
+        D.nterm = M.large ? M.nterm : M.bsz.nterm;
+        D.n_hdr = M.bsz.nhdr;
+        D.n_pair = M.bsz.npair;
+        D.n_over = M.bsz.nover;
+        D.n_over_inc = M.bsz.nover_inc;
         D.ntask = M.ntask;
         D.na = na;
         D.nc = (int32_t)M.cons.size();

@@ -802,19 +802,17 @@ static Program choose_order(int32_t nc, int32_t na, const std::vector<std::vecto
 }
 
 // ------------------------------------------------------------------------------------
-// blob writers (16-bit program for warp molecules, 32-bit for large molecules)
+// blob writers (large molecules, batched molecules)
 // ------------------------------------------------------------------------------------
-template <class IdxT>
 static ProgLayout layout_for(const MolHost& M) {
-    return prog_layout<IdxT>((uint32_t)M.atoms.size(), (uint32_t)M.cons.size(), (uint32_t)M.ntask,
+    return prog_layout<uint32_t>((uint32_t)M.atoms.size(), (uint32_t)M.cons.size(), (uint32_t)M.ntask,
                              (uint32_t)M.nterm, (uint32_t)M.nlevel, (uint32_t)M.n_seg, (uint32_t)M.n_sept,
-                             (uint32_t)M.n_cent, sizeof(IdxT) == 4 ? (uint32_t)M.pprog_bytes : 0u);
+                             (uint32_t)M.n_cent, (uint32_t)M.pprog_bytes);
 }
 
-template <class IdxT>
 static void write_blob(uint8_t* dst, const MolHost& M, const Program& P) {
-    constexpr bool kCompact = sizeof(IdxT) == 2;
-    const ProgLayout L = layout_for<IdxT>(M);
+    using IdxT = uint32_t;
+    const ProgLayout L = layout_for(M);
     std::memset(dst, 0, L.bytes);
     auto* seg = reinterpret_cast<SegRow*>(dst + L.seg);
     for (int32_t g = 0; g <= P.n_seg; ++g) seg[g] = SegRow{P.seg_piv[g], P.seg_lvl[g], P.seg_atom[g]};
@@ -851,54 +849,130 @@ static void write_blob(uint8_t* dst, const MolHost& M, const Program& P) {
         inc[fillp[con[p].i]++] = (IdxT)((uint32_t)p << 1);
         inc[fillp[con[p].j]++] = (IdxT)(((uint32_t)p << 1) | 1u);
     }
-    if constexpr (kCompact) {  // the local atom of each atom slot (ascending global order)
-        auto* aslot = reinterpret_cast<IdxT*>(dst + L.atom_off);
-        for (int32_t a = 0; a < na; ++a) aslot[M.aperm.empty() ? a : M.aperm[a]] = (IdxT)a;
-    }
     auto term_of = [&](size_t k) { return TermOf<IdxT>::make(P.terms[k].l, P.terms[k].u, P.terms[k].m); };
-    if constexpr (kCompact) {
-        // task words; terms thread by thread (thread r of the molecule's team of M.team
-        // threads owns t0 + r + M.team k of every level), each thread's terms in level order
-        auto* tasks = reinterpret_cast<uint32_t*>(dst + L.tasks);
-        auto* lane_term = reinterpret_cast<IdxT*>(dst + L.lane_term);
-        const int32_t ntask = (int32_t)P.tasks.size() - 1;
-        for (int32_t t = 0; t < ntask; ++t) {
-            const TaskW& w = P.tasks[t];
-            const uint32_t nt = P.tasks[t + 1].tstart - w.tstart;
-            tasks[t] = TaskWord::make(w.row, w.col, w.atomsign >> 1, w.atomsign & 1u, nt);
-        }
-        size_t o = 0;
-        const int32_t nl = (int32_t)P.lvl_task.size() - 1;
-        const int32_t team = M.team;
-        for (int32_t r = 0; r < team; ++r) {
-            lane_term[r] = (IdxT)o;
-            for (int32_t l = 0; l < nl; ++l) {
-                const int32_t t0 = P.lvl_task[l], t1 = P.lvl_task[l + 1];
-                for (int32_t t = t0 + r; t < t1; t += team)
-                    for (uint32_t k = P.tasks[t].tstart; k < P.tasks[t + 1].tstart; ++k) terms[o++] = term_of(k);
-            }
-        }
-    } else {
-        auto* tasks = reinterpret_cast<Task<IdxT>*>(dst + L.tasks);
-        const IdxT no_atom = (IdxT)~(IdxT)0;
-        for (size_t t = 0; t < P.tasks.size(); ++t) {
-            const TaskW& w = P.tasks[t];
-            tasks[t].row = (IdxT)w.row;
-            tasks[t].col = (IdxT)w.col;
-            tasks[t].atomsign = w.atomsign == kNoAtom32 ? no_atom : (IdxT)w.atomsign;  // sentinel
-            tasks[t].tstart = (IdxT)w.tstart;
-        }
-        for (size_t k = 0; k < P.terms.size(); ++k) terms[k] = term_of(k);
-        if (P.n_seg > 1) {
-            std::memcpy(dst + L.sep_info, P.sep_info.data(), P.sep_info.size() * sizeof(SepInfo));
-            std::memcpy(dst + L.cptr, P.cptr.data(), P.cptr.size() * sizeof(int32_t));
-            std::memcpy(dst + L.cent, P.cent.data(), P.cent.size() * sizeof(Contrib));
-            if (M.pprog_bytes > 0) {
-                std::memcpy(dst + L.pprog_off, P.pprog_off.data(), P.pprog_off.size() * sizeof(uint32_t));
-                std::memcpy(dst + L.pprog, P.pprog.data(), P.pprog.size());
-            }
+    auto* tasks = reinterpret_cast<Task<IdxT>*>(dst + L.tasks);
+    const IdxT no_atom = (IdxT)~(IdxT)0;
+    for (size_t t = 0; t < P.tasks.size(); ++t) {
+        const TaskW& w = P.tasks[t];
+        tasks[t].row = (IdxT)w.row;
+        tasks[t].col = (IdxT)w.col;
+        tasks[t].atomsign = w.atomsign == kNoAtom32 ? no_atom : (IdxT)w.atomsign;  // sentinel
+        tasks[t].tstart = (IdxT)w.tstart;
+    }
+    for (size_t k = 0; k < P.terms.size(); ++k) terms[k] = term_of(k);
+    if (P.n_seg > 1) {
+        std::memcpy(dst + L.sep_info, P.sep_info.data(), P.sep_info.size() * sizeof(SepInfo));
+        std::memcpy(dst + L.cptr, P.cptr.data(), P.cptr.size() * sizeof(int32_t));
+        std::memcpy(dst + L.cent, P.cent.data(), P.cent.size() * sizeof(Contrib));
+        if (M.pprog_bytes > 0) {
+            std::memcpy(dst + L.pprog_off, P.pprog_off.data(), P.pprog_off.size() * sizeof(uint32_t));
+            std::memcpy(dst + L.pprog, P.pprog.data(), P.pprog.size());
         }
     }
+}
+
+// Sizes of a batched molecule's program: off-diagonal pairs, items with terms (pivots, and pairs
+// U[j,q], L[q,j], whose tasks have the same earlier pivots) and their completed terms, atoms
+// of more than four constraints.
+static BatchSizes batch_sizes_of(const MolHost& M, const Program& P) {
+    BatchSizes z{(int32_t)M.atoms.size(), (int32_t)M.cons.size(), 0, P.nlevel, 0, 0, 0, 0};
+    auto item = [&](int32_t t) {
+        const int32_t n = (int32_t)(P.tasks[t + 1].tstart - P.tasks[t].tstart);
+        z.nhdr += n > 0 ? 1 : 0;
+        z.nterm += (n + 1) & ~1;
+    };
+    for (int32_t p = 0; p < z.nc; ++p) {
+        item(P.diag_task[p]);
+        for (size_t k = 0; k < P.up[p].size(); ++k) item(P.ustart[p] + (int32_t)k);
+        z.npair += (int32_t)P.up[p].size();
+    }
+    std::vector<int32_t> deg(z.na, 0);
+    for (int32_t c = 0; c < z.nc; ++c) {
+        ++deg[M.ci[c]];
+        ++deg[M.cj[c]];
+    }
+    for (int32_t a = 0; a < z.na; ++a)
+        if (deg[a] > 4) {  // a prefix: local atoms are ordered by decreasing degree
+            z.nover = a + 1;
+            z.nover_inc += deg[a] - 4;
+        }
+    return z;
+}
+
+static void write_batch_blob(uint8_t* dst, const MolHost& M, const Program& P) {
+    const BatchSizes& z = M.bsz;
+    const BatchLayout L = batch_layout(z);
+    std::memset(dst, 0, L.bytes);
+    auto u16 = [&](uint32_t off) { return reinterpret_cast<uint16_t*>(dst + off); };
+    auto u32 = [&](uint32_t off) { return reinterpret_cast<uint32_t*>(dst + off); };
+    std::vector<int32_t> pair0(z.nc + 1, 0);  // first pair of each pivot
+    for (int32_t p = 0; p < z.nc; ++p) pair0[p + 1] = pair0[p] + (int32_t)P.up[p].size();
+    std::vector<std::vector<uint32_t>> inc(z.na);
+    for (int32_t p = 0; p < z.nc; ++p) {
+        const int32_t c = P.pos_con[p];
+        u32(L.con)[p] = (uint32_t)M.ci[c] | ((uint32_t)M.cj[c] << 16);
+        u32(L.con_gid)[p] = (uint32_t)M.cons[c];
+        inc[M.ci[c]].push_back((uint32_t)p << 1);
+        inc[M.cj[c]].push_back(((uint32_t)p << 1) | 1u);
+        const auto& up = P.up[p];
+        auto q = [&](size_t k) { return k < up.size() ? (uint32_t)up[k] : 0u; };
+        u32(L.back)[2 * p] = (uint32_t)pair0[p] | ((uint32_t)up.size() << 12) | (q(0) << 20);
+        u32(L.back)[2 * p + 1] = q(1) | (q(2) << 8) | (q(3) << 16);
+        for (size_t k = 0; k < up.size(); ++k) {
+            const TaskW& w = P.tasks[P.ustart[p] + (int32_t)k];
+            u32(L.pairs)[pair0[p] + (int32_t)k] = PairWord::make(w.row, w.col, w.atomsign);
+        }
+    }
+    int32_t o = 0;
+    for (int32_t a = 0; a < z.na; ++a) {
+        for (size_t k = 0; k < 4; ++k) u16(L.inc4)[4 * a + k] = (uint16_t)(k < inc[a].size() ? inc[a][k] : kNoInc);
+        if (a >= z.nover) continue;
+        u16(L.over_ptr)[a] = (uint16_t)o;
+        for (size_t k = 4; k < inc[a].size(); ++k) u16(L.over)[o++] = (uint16_t)inc[a][k];
+        u16(L.over_ptr)[a + 1] = (uint16_t)o;
+    }
+    for (int32_t a = 0; a < z.na; ++a) u16(L.aslot)[M.aperm.empty() ? a : M.aperm[a]] = (uint16_t)a;
+    // items with terms, level by level; the terms of pair (p, q) are those of its task U[p,q],
+    // (L[p,m], U[m,q], m), as the pairs (m, p) and (m, q)
+    const uint32_t pbase = (uint32_t)batch_pivot_base(z.na, z.nc, z.npair), zero = pbase + (uint32_t)z.nc;
+    struct Item { uint32_t slot; int32_t task; bool diag; uint32_t n; };
+    std::vector<Item> items;
+    BatchHead* H = reinterpret_cast<BatchHead*>(dst);
+    H->wide32 = H->wide16 = 1;
+    H->wide_piv = 0;
+    uint32_t nh = 0, e = 0;
+    for (int32_t l = 0; l < z.nlevel; ++l) {
+        u16(L.lvl_piv)[l] = (uint16_t)P.lvl_piv[l];
+        u16(L.lvl_hdr)[l] = (uint16_t)nh;
+        items.clear();
+        for (int32_t p = P.lvl_piv[l]; p < P.lvl_piv[l + 1]; ++p) {
+            auto add = [&](uint32_t slot, int32_t task, bool diag) {
+                const uint32_t n = P.tasks[task + 1].tstart - P.tasks[task].tstart;
+                if (n > 0) items.push_back(Item{slot, task, diag, n});
+            };
+            add(pbase + (uint32_t)p, P.diag_task[p], true);
+            for (size_t k = 0; k < P.up[p].size(); ++k)
+                add((uint32_t)(pair0[p] + (int32_t)k), P.ustart[p] + (int32_t)k, false);
+        }
+        std::stable_sort(items.begin(), items.end(), [](const Item& x, const Item& y) { return x.n > y.n; });
+        for (const Item& it : items) {
+            u32(L.hdr)[nh++] = HeadWord::make(it.slot, it.diag, (it.n + 1) / 2, e / 2);
+            uint32_t m = 0;
+            for (uint32_t x = P.tasks[it.task].tstart; x < P.tasks[it.task + 1].tstart; ++x) {
+                m = P.terms[x].m;
+                const uint32_t us = (uint32_t)P.ustart[m], nu = (uint32_t)P.up[m].size();
+                const uint32_t a = (uint32_t)pair0[m] + (P.terms[x].l - us - nu);
+                const uint32_t b = (uint32_t)pair0[m] + (P.terms[x].u - us);
+                u32(L.terms)[e++] = TermWord::make(a, b, m);
+            }
+            if (it.n & 1u) u32(L.terms)[e++] = TermWord::make(zero, zero, m);
+        }
+        if (items.size() > 32) H->wide32 = (uint16_t)(l + 1);
+        if (items.size() > 16) H->wide16 = (uint16_t)(l + 1);
+        if (P.lvl_piv[l + 1] - P.lvl_piv[l] > 32) H->wide_piv = (uint16_t)(l + 1);
+    }
+    u16(L.lvl_piv)[z.nlevel] = (uint16_t)P.lvl_piv[z.nlevel];
+    u16(L.lvl_hdr)[z.nlevel] = (uint16_t)nh;
 }
 
 // Batched molecules: relabel the local atoms in order of decreasing degree (number of
@@ -927,13 +1001,17 @@ static void relabel_atoms_by_degree(MolHost& M, Program& P) {
     }
 }
 
-// true if a program fits the compact (warp) encoding: task words hold at most
-// TaskWord::kMaxTerms terms, term and slot indices fit their fields
+// true if a program fits the batched kernel's encoding: value slots, terms per item (pivots and
+// entries of U; those of L share their terms) and term pairs fit their fields
 static bool fits_compact(const Program& P) {
-    if (P.tasks.size() >= kCompactMaxSlots || P.terms.size() > kCompactMaxTerms) return false;
-    for (size_t t = 0; t + 1 < P.tasks.size(); ++t)
-        if (P.tasks[t + 1].tstart - P.tasks[t].tstart > TaskWord::kMaxTerms) return false;
-    return true;
+    if (P.tasks.size() >= kCompactMaxSlots) return false;
+    uint32_t term_pairs = 0;
+    for (size_t t = 0; t + 1 < P.tasks.size(); ++t) {
+        const uint32_t n = P.tasks[t + 1].tstart - P.tasks[t].tstart;
+        if (n > HeadWord::kMaxTerms) return false;
+        if (P.tasks[t].row <= P.tasks[t].col) term_pairs += (n + 1) / 2;
+    }
+    return term_pairs < HeadWord::kMaxPairs;
 }
 
 // ------------------------------------------------------------------------------------
@@ -1026,7 +1104,7 @@ ilves_status plan_topology(ilves_topology* T, int32_t n_atoms, int32_t n_c, cons
         int64_t batched = 0, small = 0, n_batched = 0;
         for (int32_t m = 0; m < n_mol; ++m) {
             const int64_t na = (int64_t)T->mols[m].atoms.size(), nc = (int64_t)T->mols[m].cons.size();
-            if (nc > warp_limit || nc >= (int64_t)kCompactMaxConstraints || na > (int64_t)TaskWord::kMaxAtom) continue;
+            if (nc > warp_limit || nc >= (int64_t)kCompactMaxConstraints || na > (int64_t)PairWord::kMaxAtom) continue;
             batched += na;
             ++n_batched;
             if (na <= kDefaultNarrowAtoms) small += na;
@@ -1058,7 +1136,7 @@ ilves_status plan_topology(ilves_topology* T, int32_t n_atoms, int32_t n_c, cons
             std::sort(v.begin(), v.end());
             v.erase(std::unique(v.begin(), v.end()), v.end());
         }
-        M.large = nc > warp_limit || nc >= (int32_t)kCompactMaxConstraints || na > (int32_t)TaskWord::kMaxAtom;
+        M.large = nc > warp_limit || nc >= (int32_t)kCompactMaxConstraints || na > (int32_t)PairWord::kMaxAtom;
         const int32_t part_min = o.partition_min_constraints > 0 ? o.partition_min_constraints : 4096;
         if (nc >= part_min && o.overlap > 0) {
             // overlapping domains: parts of ~part_size constraints, each domain widened by
@@ -1178,7 +1256,10 @@ ilves_status plan_topology(ilves_topology* T, int32_t n_atoms, int32_t n_c, cons
             M.team = kSlotThreads;
             *P = choose_order(nc, na, adj, M.ci, M.cj, o, 1024);
         }
-        if (!M.large) relabel_atoms_by_degree(M, *P);
+        if (!M.large) {
+            relabel_atoms_by_degree(M, *P);
+            M.bsz = batch_sizes_of(M, *P);
+        }
         M.nlevel = P->nlevel;
         M.ntask = (int32_t)P->tasks.size() - 1;
         M.nterm = (int32_t)P->terms.size();
@@ -1192,7 +1273,7 @@ ilves_status plan_topology(ilves_topology* T, int32_t n_atoms, int32_t n_c, cons
 int64_t program_blob_bytes(const ilves_topology* T, int32_t m) {
     const MolHost& M = T->mols[m];
     if (M.opm) return (int64_t)T->progs[m]->opm_blob.size();
-    return M.large ? layout_for<uint32_t>(M).bytes : layout_for<uint16_t>(M).bytes;
+    return M.large ? layout_for(M).bytes : batch_layout(M.bsz).bytes;
 }
 
 void program_write_blob(const ilves_topology* T, int32_t m, uint8_t* dst) {
@@ -1200,9 +1281,9 @@ void program_write_blob(const ilves_topology* T, int32_t m, uint8_t* dst) {
     if (M.opm)
         std::memcpy(dst, T->progs[m]->opm_blob.data(), T->progs[m]->opm_blob.size());
     else if (M.large)
-        write_blob<uint32_t>(dst, M, *T->progs[m]);
+        write_blob(dst, M, *T->progs[m]);
     else
-        write_blob<uint16_t>(dst, M, *T->progs[m]);
+        write_batch_blob(dst, M, *T->progs[m]);
 }
 
 void program_export(const ilves_topology* T, int32_t m, int32_t* pos_gid, int32_t* level,
@@ -1287,10 +1368,8 @@ void free_programs(ilves_topology* T) {
 // bytes of one molecule's shared-memory slice for a precision mode
 uint32_t footprint(const MolHost& M, int mode) {
     const uint32_t lp = mode == ILVES_PREC_FP64 ? 8u : 4u;
-    const ProgLayout L = layout_for<uint16_t>(M);
-    const StateLayout S = state_layout((uint32_t)M.atoms.size(), (uint32_t)M.cons.size(), (uint32_t)M.ntask,
-                                       lp, mode == ILVES_PREC_MIXED_DF);
-    return L.staged + S.bytes;
+    return batch_layout(M.bsz).staged + batch_state((uint32_t)M.bsz.na, (uint32_t)M.bsz.nc, (uint32_t)M.bsz.npair, lp,
+                                                    mode == ILVES_PREC_MIXED_DF).bytes;
 }
 
 // Slot schedule of the batched kernel.  Molecules of each class (96-thread teams, and the
