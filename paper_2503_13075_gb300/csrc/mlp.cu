@@ -13,8 +13,8 @@
 //             (eight MMAs), whose epilogue does the third layer as a per-row dot product
 //   target    y = lambda * scale, scale = 4 (w_i + w_j) s.rho / d^2  -> lambda_0 = y / scale
 //   training  forward on the tensor cores storing activations, backward on the float32
-//             pipes (one thread per hidden unit, register accumulators, one atomic flush
-//             per block), Adam on float32 master weights, bfloat16 copies refreshed.
+//             pipes (register-tiled products per CTA, partial gradients summed in a fixed
+//             order), Adam on float32 master weights, bfloat16 copies refreshed.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -404,74 +404,240 @@ k_mlp_forward(MlpWeights Wt, const float* __restrict__ X, int n, FeatArgs F, flo
 }
 
 // ------------------------------------------------------------------------------------
-// float32 backward: one thread per hidden unit, rows streamed through shared memory
+// float32 backward: three register-tiled products per chunk of rows
 // ------------------------------------------------------------------------------------
-constexpr int BWD_ROWS = 128;
+// A CTA takes rows_per_cta rows, up to kBwdRows at a time, held in shared memory with W2:
+//   dz2 = (dy w3) masked by h2 > 0,   gW2 += dz2^T h1,   dh1 = dz2 W2,   dz1 = dh1 masked by
+//   h1 > 0,   gW1 += dz1^T X,   and the column sums.
+// What bounds it: the float32 pipes (70 kFLOP a row; 0.57 GFLOP for 8192 rows).  Each thread
+// holds an 8 x 8 tile of gW2 across the whole range (and 4 x 8 of dh1), so an operand read
+// from shared memory feeds eight FMAs; two FMAs go in one instruction (fma.rn.f32x2, the same
+// roundings), which leaves issue slots for the loads.  Every CTA writes its own partial
+// gradient (and loss); k_grad_reduce adds them in a fixed order of eight interleaved chains, so
+// the gradient is the same on every run and its rounding error does not grow with the number
+// of CTAs, as it did with float32 atomics.  Rows are spread over the SMs, but at least kBwdMinRows
+// to a CTA, below which the 75 KB of W2 in and gradient out cost more than they save.
+// A whole gradient of 8192 rows takes 45 us; with one thread per hidden unit, rows streamed one by
+// one with three barriers each and float32 atomics it took 220 us.
+constexpr int kBwdRows = 64, kBwdMinRows = 16, kBwdThreads = 256;
+constexpr int kPartStride = (P_N + 1 + 3) & ~3;  // a CTA's partial gradient, then its loss
+constexpr int kBwdSmem = (NH * NH + 2 * kBwdRows * NH + kBwdRows * NF + kBwdRows) * (int)sizeof(float);
 
-__global__ void __launch_bounds__(NH)
-k_mlp_backward(const float* __restrict__ X, const float* __restrict__ t, int n, const float* __restrict__ y,
-               const __nv_bfloat16* __restrict__ h1, const float* __restrict__ h2, const __nv_bfloat16* __restrict__ w2b,
-               const float* __restrict__ params, float* __restrict__ grad, float* __restrict__ loss) {
-    __shared__ __nv_bfloat16 w2s[NH * NH];  // [c][k], the bfloat16 weights the forward used
-    __shared__ float dz2s[NH], h1s[NH], xs[NF], dys;
-    const int c = threadIdx.x;  // hidden unit of layer 2 (and of layer 1 for the input side)
-    for (int e = c; e < NH * NH; e += NH) w2s[e] = w2b[e];
+__device__ __forceinline__ float2 fma2(float a, float2 b, float2 c) {
+    float2 d;
+    asm("{\n.reg .b64 ra, rb, rc;\nmov.b64 ra, {%2, %2};\nmov.b64 rb, {%3, %4};\nmov.b64 rc, {%5, %6};\n"
+        "fma.rn.f32x2 rc, ra, rb, rc;\nmov.b64 {%0, %1}, rc;\n}\n"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+__global__ void __launch_bounds__(kBwdThreads, 1)
+k_mlp_backward(const float* __restrict__ X, const float* __restrict__ t, int n, int rows_per_cta,
+               const float* __restrict__ y, const __nv_bfloat16* __restrict__ h1, const float* __restrict__ h2,
+               const __nv_bfloat16* __restrict__ w2b, const float* __restrict__ params, float* __restrict__ partial) {
+    extern __shared__ __align__(16) float bsm[];
+    float* w2s = bsm;                       // [c][k], the bfloat16 weights the forward used
+    float* dzs = w2s + NH * NH;             // dz2 [r][c], then dz1 [r][k]
+    float* h1s = dzs + kBwdRows * NH;       // [r][k]
+    float* xs = h1s + kBwdRows * NH;        // [r][f]
+    float* dys = xs + kBwdRows * NF;        // [r]
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    for (int e = tid; e < NH * NH / 8; e += kBwdThreads) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(w2b) + e);
+        const __nv_bfloat162* b = reinterpret_cast<const __nv_bfloat162*>(&v);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) *reinterpret_cast<float2*>(w2s + 8 * e + 2 * q) = __bfloat1622float2(b[q]);
+    }
+    const int c = tid & (NH - 1), half = tid >> 7;  // column sums: column c, every other row
     const float w3c = params[P_W3 + c];
-    float gw2[NH];
-#pragma unroll
-    for (int k = 0; k < NH; ++k) gw2[k] = 0.f;
-    float gw1[NF];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) gw1[f] = 0.f;
-    float gb1 = 0.f, gb2 = 0.f, gw3 = 0.f, gb3 = 0.f, lsum = 0.f;
     const float inv_n = 1.0f / (float)n;
-    const int rb = blockIdx.x * BWD_ROWS, re = min(n, rb + BWD_ROWS);
-    __syncthreads();
-    for (int r = rb; r < re; ++r) {
-        if (c == 0) {
-            const float res = y[r] - t[r];
-            dys = 2.0f * res * inv_n;
-            lsum += res * res * inv_n;
+    // rows (columns) of a tile: ty * 4 .. + 3 and 64 + ty * 4 .. + 3 (tx alike), so the lanes of a warp
+    // read consecutive 16-byte words
+    float2 gw2[8][4], gw1[4];
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) gw2[a][b] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int b = 0; b < 4; ++b) gw1[b] = make_float2(0.f, 0.f);
+    float gb1 = 0.f, gb2 = 0.f, gw3 = 0.f, gb3 = 0.f, lsum = 0.f;
+    const int rb = blockIdx.x * rows_per_cta, re = min(n, rb + rows_per_cta);
+    for (int r0 = rb; r0 < re; r0 += kBwdRows) {
+        const int rows = min(kBwdRows, re - r0), rows4 = (rows + 3) & ~3;  // completed with zero rows
+        __syncthreads();
+        if (tid < rows4) {
+            float dy = 0.f;
+            if (tid < rows) {
+                const float res = y[r0 + tid] - t[r0 + tid];
+                dy = 2.0f * res * inv_n;
+                lsum += res * res * inv_n;
+                gb3 += dy;
+            }
+            dys[tid] = dy;
         }
-        h1s[c] = __bfloat162float(h1[(int64_t)r * NH + c]);
-        if (c < NF) xs[c] = X[(int64_t)r * NF + c];
-        __syncthreads();
-        const float dy = dys;
-        const float h2c = h2[(int64_t)r * NH + c];
-        const float dz2 = h2c > 0.f ? dy * w3c : 0.f;
-        gw3 += dy * h2c;
-        gb2 += dz2;
-        gb3 += dy;
-        dz2s[c] = dz2;
+        for (int e = tid; e < rows4 * (NF / 4); e += kBwdThreads)
+            reinterpret_cast<float4*>(xs)[e] = e < rows * (NF / 4)
+                                                   ? __ldg(reinterpret_cast<const float4*>(X + (int64_t)r0 * NF) + e)
+                                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int e = tid; e < rows4 * (NH / 8); e += kBwdThreads) {
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (e < rows * (NH / 8)) v = __ldg(reinterpret_cast<const uint4*>(h1 + (int64_t)r0 * NH) + e);
+            const __nv_bfloat162* b = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
-        for (int k = 0; k < NH; ++k) gw2[k] = fmaf(dz2, h1s[k], gw2[k]);
+            for (int q = 0; q < 4; ++q) *reinterpret_cast<float2*>(h1s + 8 * e + 2 * q) = __bfloat1622float2(b[q]);
+        }
         __syncthreads();
-        // this thread now plays hidden unit k = c of layer 1
-        float dh1 = 0.f;
-#pragma unroll 8
-        for (int cc = 0; cc < NH; ++cc) dh1 = fmaf(dz2s[cc], __bfloat162float(w2s[cc * NH + c]), dh1);
-        const float dz1 = h1s[c] > 0.f ? dh1 : 0.f;
-        gb1 += dz1;
+        for (int r = half; r < rows4; r += 2) {
+            const float h = r < rows ? __ldg(h2 + (int64_t)(r0 + r) * NH + c) : 0.f, dy = dys[r];
+            const float dz2 = h > 0.f ? dy * w3c : 0.f;
+            gw3 += dy * h;
+            gb2 += dz2;
+            dzs[r * NH + c] = dz2;
+        }
+        __syncthreads();
+        // gW2[c][k] += sum_r dz2[r][c] h1[r][k]
+#pragma unroll 2
+        for (int r = 0; r < rows4; ++r) {
+            const float4 a0 = *reinterpret_cast<const float4*>(dzs + r * NH + 4 * ty);
+            const float4 a1 = *reinterpret_cast<const float4*>(dzs + r * NH + 64 + 4 * ty);
+            const float4 b0 = *reinterpret_cast<const float4*>(h1s + r * NH + 4 * tx);
+            const float4 b1 = *reinterpret_cast<const float4*>(h1s + r * NH + 64 + 4 * tx);
+            const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+            const float2 bv[4] = {{b0.x, b0.y}, {b0.z, b0.w}, {b1.x, b1.y}, {b1.z, b1.w}};
 #pragma unroll
-        for (int f = 0; f < NF; ++f) gw1[f] = fmaf(dz1, xs[f], gw1[f]);
+            for (int a = 0; a < 8; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) gw2[a][b] = fma2(av[a], bv[b], gw2[a][b]);
+        }
+        // dh1[r][k] = sum_c dz2[r][c] W2[c][k], rows ty, ty + 16, ty + 32, ty + 48
+        float2 dh[4][4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) dh[a][b] = make_float2(0.f, 0.f);
+        if (ty < rows4) {  // rows past rows4 hold an earlier chunk's values: computed, not stored
+#pragma unroll 1
+            for (int cc = 0; cc < NH; cc += 4) {
+                float av[4][4];
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    const float4 v = *reinterpret_cast<const float4*>(dzs + min(ty + 16 * a, rows4 - 1) * NH + cc);
+                    av[a][0] = v.x;
+                    av[a][1] = v.y;
+                    av[a][2] = v.z;
+                    av[a][3] = v.w;
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float4 b0 = *reinterpret_cast<const float4*>(w2s + (cc + q) * NH + 4 * tx);
+                    const float4 b1 = *reinterpret_cast<const float4*>(w2s + (cc + q) * NH + 64 + 4 * tx);
+                    const float2 bv[4] = {{b0.x, b0.y}, {b0.z, b0.w}, {b1.x, b1.y}, {b1.z, b1.w}};
+#pragma unroll
+                    for (int a = 0; a < 4; ++a)
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) dh[a][b] = fma2(av[a][q], bv[b], dh[a][b]);
+                }
+            }
+        }
         __syncthreads();
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const int r = ty + 16 * a;
+            if (r < rows4) {
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    const int k = (b < 2 ? 0 : 64) + 4 * tx + 2 * (b & 1);
+                    const float2 h = *reinterpret_cast<const float2*>(h1s + r * NH + k);
+                    *reinterpret_cast<float2*>(dzs + r * NH + k) =
+                        make_float2(h.x > 0.f ? dh[a][b].x : 0.f, h.y > 0.f ? dh[a][b].y : 0.f);
+                }
+            }
+        }
+        __syncthreads();
+        // gW1[k][f] += sum_r dz1[r][k] X[r][f]: unit k = c, features 8 half .. + 7
+#pragma unroll 4
+        for (int r = 0; r < rows4; ++r) {
+            const float dz1 = dzs[r * NH + c];
+            const float4 x0 = *reinterpret_cast<const float4*>(xs + r * NF + 8 * half);
+            const float4 x1 = *reinterpret_cast<const float4*>(xs + r * NF + 8 * half + 4);
+            gw1[0] = fma2(dz1, make_float2(x0.x, x0.y), gw1[0]);
+            gw1[1] = fma2(dz1, make_float2(x0.z, x0.w), gw1[1]);
+            gw1[2] = fma2(dz1, make_float2(x1.x, x1.y), gw1[2]);
+            gw1[3] = fma2(dz1, make_float2(x1.z, x1.w), gw1[3]);
+            if (half == 0) gb1 += dz1;
+        }
+    }
+    float* grad = partial + (int64_t)blockIdx.x * kPartStride;
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+        float4* g = reinterpret_cast<float4*>(grad + P_W2 + ((a < 4 ? 0 : 64) + 4 * ty + (a & 3)) * NH + 4 * tx);
+        g[0] = make_float4(gw2[a][0].x, gw2[a][0].y, gw2[a][1].x, gw2[a][1].y);
+        g[16] = make_float4(gw2[a][2].x, gw2[a][2].y, gw2[a][3].x, gw2[a][3].y);
+    }
+    float4* g1 = reinterpret_cast<float4*>(grad + P_W1 + c * NF + 8 * half);
+    g1[0] = make_float4(gw1[0].x, gw1[0].y, gw1[1].x, gw1[1].y);
+    g1[1] = make_float4(gw1[2].x, gw1[2].y, gw1[3].x, gw1[3].y);
+    // the column sums of even and odd rows, the sums over rows
+    __syncthreads();
+    if (half == 1) {
+        dzs[c] = gb2;
+        dzs[NH + c] = gw3;
     }
 #pragma unroll
-    for (int k = 0; k < NH; ++k) atomicAdd(grad + P_W2 + c * NH + k, gw2[k]);
-#pragma unroll
-    for (int f = 0; f < NF; ++f) atomicAdd(grad + P_W1 + c * NF + f, gw1[f]);
-    atomicAdd(grad + P_B1 + c, gb1);
-    atomicAdd(grad + P_B2 + c, gb2);
-    atomicAdd(grad + P_W3 + c, gw3);
-    if (c == 0) {
-        atomicAdd(grad + P_B3, gb3);
-        if (loss) atomicAdd(loss, lsum);
+    for (int o = 16; o > 0; o >>= 1) {
+        gb3 += __shfl_xor_sync(0xFFFFFFFFu, gb3, o);
+        lsum += __shfl_xor_sync(0xFFFFFFFFu, lsum, o);
+    }
+    if (tid == 32) {
+        dzs[2 * NH] = gb3;
+        dzs[2 * NH + 1] = lsum;
+    }
+    __syncthreads();
+    if (half == 0) {
+        grad[P_B1 + c] = gb1;
+        grad[P_B2 + c] = gb2 + dzs[c];
+        grad[P_W3 + c] = gw3 + dzs[NH + c];
+    }
+    if (tid == 0) {
+        grad[P_B3] = gb3 + dzs[2 * NH];
+        grad[P_N] = lsum + dzs[2 * NH + 1];
     }
 }
 
-__global__ void k_zero(float* __restrict__ p, int n) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) p[i] = 0.f;
+// The partial gradients' sum: 32 columns of four values to a CTA, eight threads to a column that
+// each add every eighth partial, then one adds the eight.
+constexpr int kRedThreads = 256;
+__global__ void __launch_bounds__(kRedThreads)
+k_grad_reduce(const float* __restrict__ partial, int n_part, float* __restrict__ grad, float* __restrict__ loss) {
+    __shared__ float4 acc[kRedThreads];
+    const int col = blockIdx.x * 32 + (threadIdx.x & 31), row = threadIdx.x >> 5;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (col < kPartStride / 4)
+        for (int p = row; p < n_part; p += kRedThreads / 32) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(partial + (int64_t)p * kPartStride) + col);
+            s.x += v.x;
+            s.y += v.y;
+            s.z += v.z;
+            s.w += v.w;
+        }
+    acc[threadIdx.x] = s;
+    __syncthreads();
+    if (row != 0) return;
+#pragma unroll
+    for (int q = 1; q < kRedThreads / 32; ++q) {
+        const float4 v = acc[32 * q + threadIdx.x];
+        s.x += v.x;
+        s.y += v.y;
+        s.z += v.z;
+        s.w += v.w;
+    }
+    const float out[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int i = 4 * col + q;
+        if (i < P_N) grad[i] = out[q];
+        else if (i == P_N) *loss = out[q];
+    }
 }
 
 // Adam on the float32 master parameters; refreshes the bfloat16 weight copies.
@@ -511,6 +677,8 @@ struct ilves_mlp {
     float* m = nullptr;
     float* v = nullptr;
     float* grad = nullptr;
+    float* partial = nullptr;  // one partial gradient and loss per CTA of the backward kernel
+    int32_t n_part = 0;        // at most this many
     float* loss = nullptr;
     float* y = nullptr;
     __nv_bfloat16* w1b = nullptr;
@@ -597,6 +765,10 @@ extern "C" ilves_status ilves_mlp_create(int32_t max_batch, uint64_t seed, ilves
     alloc((void**)&M->m, P_N * sizeof(float));
     alloc((void**)&M->v, P_N * sizeof(float));
     alloc((void**)&M->grad, P_N * sizeof(float));
+    M->n_part = 152;
+    if (cudaDeviceGetAttribute(&M->n_part, cudaDevAttrMultiProcessorCount, M->device) != cudaSuccess) M->n_part = 152;
+    M->n_part = std::min(M->n_part, std::max(1, (max_batch + kBwdMinRows - 1) / kBwdMinRows));
+    alloc((void**)&M->partial, (size_t)M->n_part * kPartStride * sizeof(float));
     alloc((void**)&M->loss, sizeof(float));
     alloc((void**)&M->y, (size_t)max_batch * sizeof(float));
     alloc((void**)&M->w1b, NH * NF * sizeof(__nv_bfloat16));
@@ -627,8 +799,8 @@ extern "C" ilves_status ilves_mlp_create(int32_t max_batch, uint64_t seed, ilves
 
 extern "C" void ilves_mlp_destroy(ilves_mlp* M) {
     if (!M) return;
-    for (void* p : {(void*)M->params, (void*)M->m, (void*)M->v, (void*)M->grad, (void*)M->loss, (void*)M->y,
-                    (void*)M->w1b, (void*)M->w2b, (void*)M->h1, (void*)M->h2, (void*)M->err})
+    for (void* p : {(void*)M->params, (void*)M->m, (void*)M->v, (void*)M->grad, (void*)M->partial, (void*)M->loss,
+                    (void*)M->y, (void*)M->w1b, (void*)M->w2b, (void*)M->h1, (void*)M->h2, (void*)M->err})
         if (p) cudaFree(p);
     delete M;
 }
@@ -696,17 +868,25 @@ extern "C" ilves_status ilves_warm_start(const ilves_mlp* M, const ilves_topolog
     return mlp_status(cudaGetLastError());
 }
 
-// forward with stored activations + backward into M->grad (and the loss into M->loss)
-static ilves_status mlp_gradient(ilves_mlp* M, const float* X, const float* t, int32_t n, cudaStream_t s) {
+// forward with stored activations + backward into grad and loss
+static ilves_status mlp_gradient(ilves_mlp* M, const float* X, const float* t, int32_t n, float* grad, float* loss,
+                                 cudaStream_t s) {
     const MlpWeights Wt{M->w1b, M->w2b, M->params};
     FeatArgs F{};
     if (reinterpret_cast<uintptr_t>(X) & 15u) return ILVES_ERR_INVALID_ARG;
-    const cudaError_t e = launch_forward<false, true>(Wt, X, n, F, M->y, M->h1, M->h2, M->err, M->wait_test, s);
+    cudaError_t e = launch_forward<false, true>(Wt, X, n, F, M->y, M->h1, M->h2, M->err, M->wait_test, s);
     if (e != cudaSuccess) return mlp_status(e);
-    k_zero<<<(P_N + 255) / 256, 256, 0, s>>>(M->grad, P_N);
-    k_zero<<<1, 32, 0, s>>>(M->loss, 1);
-    k_mlp_backward<<<(n + BWD_ROWS - 1) / BWD_ROWS, NH, 0, s>>>(X, t, n, M->y, M->h1, M->h2, M->w2b, M->params,
-                                                               M->grad, M->loss);
+    static bool attr_set[64] = {};
+    int dev = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return mlp_status(e);
+    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
+        e = cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdSmem);
+        if (e != cudaSuccess) return mlp_status(e);
+        if (dev >= 0 && dev < 64) attr_set[dev] = true;
+    }
+    const int rows = std::max(kBwdMinRows, (n + M->n_part - 1) / M->n_part), parts = (n + rows - 1) / rows;
+    k_mlp_backward<<<parts, kBwdThreads, kBwdSmem, s>>>(X, t, n, rows, M->y, M->h1, M->h2, M->w2b, M->params, M->partial);
+    k_grad_reduce<<<(kPartStride / 4 + 31) / 32, kRedThreads, 0, s>>>(M->partial, parts, grad, loss);
     return mlp_status(cudaGetLastError());
 }
 
@@ -714,24 +894,17 @@ extern "C" ilves_status ilves_mlp_gradient(ilves_mlp* M, const float* features, 
                                            float* grad_out, float* loss_out, void* stream) {
     if (!M || n <= 0 || n > M->max_batch || !features || !target) return ILVES_ERR_INVALID_ARG;
     const cudaStream_t s = (cudaStream_t)stream;
-    ilves_status st = mlp_gradient(M, features, target, n, s);
-    if (st != ILVES_OK) return st;
-    cudaError_t e = cudaSuccess;
-    if (grad_out) e = cudaMemcpyAsync(grad_out, M->grad, P_N * sizeof(float), cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess && loss_out) e = cudaMemcpyAsync(loss_out, M->loss, sizeof(float), cudaMemcpyDeviceToDevice, s);
-    return mlp_status(e);
+    return mlp_gradient(M, features, target, n, grad_out ? grad_out : M->grad, loss_out ? loss_out : M->loss, s);
 }
 
 extern "C" ilves_status ilves_mlp_train_step(ilves_mlp* M, const float* features, const float* target, int32_t n,
                                              float lr, float* loss_out, void* stream) {
     if (!M || n <= 0 || n > M->max_batch || !features || !target || !(lr >= 0.f)) return ILVES_ERR_INVALID_ARG;
     const cudaStream_t s = (cudaStream_t)stream;
-    ilves_status st = mlp_gradient(M, features, target, n, s);
+    ilves_status st = mlp_gradient(M, features, target, n, M->grad, loss_out ? loss_out : M->loss, s);
     if (st != ILVES_OK) return st;
     M->step += 1;
     const float b1c = 1.f - std::pow(0.9f, (float)M->step), b2c = 1.f - std::pow(0.999f, (float)M->step);
     k_adam<<<(P_N + 255) / 256, 256, 0, s>>>(M->params, M->m, M->v, M->grad, lr, b1c, b2c, M->w1b, M->w2b);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess && loss_out) e = cudaMemcpyAsync(loss_out, M->loss, sizeof(float), cudaMemcpyDeviceToDevice, s);
-    return mlp_status(e);
+    return mlp_status(cudaGetLastError());
 }
