@@ -36,7 +36,8 @@ constexpr int NF = ILVES_MLP_FEATURES, NH = ILVES_MLP_HIDDEN;
 constexpr int P_W1 = 0, P_B1 = P_W1 + NH * NF, P_W2 = P_B1 + NH, P_B2 = P_W2 + NH * NH, P_W3 = P_B2 + NH,
               P_B3 = P_W3 + NH, P_N = P_B3 + 1;
 static_assert(P_N == ILVES_MLP_PARAMS, "parameter count");
-constexpr int TILE = 128;  // rows per tensor-core tile (M of the MMA), one thread per row
+constexpr int TILE = 128;  // rows per tensor-core tile (M of the MMA)
+constexpr int kFwdThreads = 2 * TILE;  // two threads to a row
 
 // ------------------------------------------------------------------------------------
 // features
@@ -48,10 +49,9 @@ struct FeatArgs {
     const double* d;
     const int32_t* con_i;
     const int32_t* con_j;
-    const int32_t* nbr;
-    const int32_t* nbr_atom;
-    float4* ws_con;    // per constraint: (s.xyz, sigma0 / d^2), (rho.xyz, d)
-    float* ws_atom;    // per atom: inverse mass
+    const int4* nbr;  // four neighbour slots: neighbour << 1 | (sign product < 0), or -1
+    float4* ws_con;   // per constraint: (s.xyz, sigma0 / d^2), (rho.xyz, d)
+    float* ws_atom;   // per atom: inverse mass
     int32_t n_c;
     int32_t n_atoms;
 };
@@ -63,8 +63,8 @@ __device__ __forceinline__ float3 sub3(float3 a, float3 b) { return make_float3(
 __device__ __forceinline__ float dot3(float3 a, float3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 
 // Prep pass: per-constraint float32 geometry and per-atom weights into the topology's
-// warm-start workspace, so the feature stage gathers 32 bytes per neighbour instead of
-// four float64 atom positions.
+// warm-start workspace, so the feature stage gathers 20 bytes per neighbour instead of four
+// float64 atom positions.
 __global__ void k_ws_prep(FeatArgs F) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < F.n_c) {
@@ -78,18 +78,22 @@ __global__ void k_ws_prep(FeatArgs F) {
     if (k < F.n_atoms) F.ws_atom[k] = narrow(F.inv_mass[k]);
 }
 
-// Features of constraint k from the workspace; `half` selects which half of the 16
-// features this lane writes (two lanes per row): half 0 = own terms + slots 0-1,
-// half 1 = slots 2-3 (the scale is produced by half 0).
-__device__ __forceinline__ void ws_features(const FeatArgs& F, int k, int half, float* f, float& scale) {
+// Features of constraint k from the workspace; `half` selects which of the 16 features this
+// thread writes (two threads per row): half 0 = own terms + slots 0-1 (neighbours at atom i),
+// half 1 = slots 2-3 (at atom j; the scale is produced by half 0).  The shared atom of a slot
+// is the half's own atom and its sign comes with the neighbour, so a neighbour costs two loads
+// in the second of two rounds.
+template <int half>
+__device__ __forceinline__ void ws_features(const FeatArgs& F, int k, float* f, float& scale) {
+    const int2 nb = __ldg(reinterpret_cast<const int2*>(F.nbr + k) + half);
     const float4 s4 = F.ws_con[2 * k], r4 = F.ws_con[2 * k + 1];
-    const int i = F.con_i[k], j = F.con_j[k];
-    const float wi = F.ws_atom[i], wj = F.ws_atom[j], W = wi + wj;
+    const float wi = F.ws_atom[F.con_i[k]], wj = F.ws_atom[F.con_j[k]], W = wi + wj;
     const float inv_w = W > 0.f ? 1.0f / W : 0.f;
-    const float dk = r4.w, inv_d2 = 1.0f / (dk * dk);
-    const float3 s = make_float3(s4.x, s4.y, s4.z), r = make_float3(r4.x, r4.y, r4.z);
-    const float sr = dot3(s, r);
+    const float dk = r4.w;
+    const float3 s = make_float3(s4.x, s4.y, s4.z);
     if (half == 0) {
+        const float3 r = make_float3(r4.x, r4.y, r4.z);
+        const float inv_d2 = 1.0f / (dk * dk), sr = dot3(s, r);
         const float3 sm = sub3(s, r);
         f[0] = s4.w;
         f[1] = sr * inv_d2 - 1.0f;
@@ -99,16 +103,15 @@ __device__ __forceinline__ void ws_features(const FeatArgs& F, int k, int half, 
     }
 #pragma unroll
     for (int qq = 0; qq < 2; ++qq) {
-        const int q = 2 * half + qq;
-        const int l = F.nbr[4 * k + q];
+        const int q = 2 * half + qq, e = qq == 0 ? nb.x : nb.y;
         float g0 = 0.f, g1 = 0.f, g2 = 0.f;
-        if (l >= 0) {
-            const int a = F.nbr_atom[4 * k + q];
-            const float4 sl4 = F.ws_con[2 * l], rl4 = F.ws_con[2 * l + 1];
-            const float sgn = ((a == i) == (a == F.con_i[l])) ? 1.f : -1.f;
-            g0 = sl4.w;
+        if (e >= 0) {
+            const int l = e >> 1;
+            const float4 rl4 = F.ws_con[2 * l + 1];
+            g0 = F.ws_con[2 * l].w;
+            const float sgn = (e & 1) ? -1.f : 1.f;
             g1 = sgn * dot3(s, make_float3(rl4.x, rl4.y, rl4.z)) / (dk * rl4.w);
-            g2 = F.ws_atom[a] * inv_w;
+            g2 = (half == 0 ? wi : wj) * inv_w;
         }
         f[4 + 3 * q] = g0;
         f[5 + 3 * q] = g1;
@@ -120,8 +123,8 @@ __global__ void k_features(FeatArgs F, float* __restrict__ feat, float* __restri
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= F.n_c) return;
     float f[NF], sc = 0.f;
-    ws_features(F, k, 0, f, sc);
-    ws_features(F, k, 1, f, sc);
+    ws_features<0>(F, k, f, sc);
+    ws_features<1>(F, k, f, sc);
 #pragma unroll
     for (int q = 0; q < NF; ++q) feat[(int64_t)k * NF + q] = f[q];
     if (scale) scale[k] = sc;
@@ -148,6 +151,12 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<const uint32_t*>(&v);
 }
+
+__device__ __forceinline__ void copy16(void* smem, const void* gmem) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem)
+                 : "memory");
+}
+__device__ __forceinline__ void copy_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 struct MlpWeights {
     const __nv_bfloat16* w1;  // [NH][NF]  (out x in) bfloat16
@@ -224,21 +233,27 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
 // 74 KB, so at most three CTAs share an SM and their tensor memory (3 x 128 of 512
 // columns) always fits
 constexpr uint32_t SM_W1 = 0, SM_W2 = SM_W1 + NH * NF * 2, SM_A1 = SM_W2 + NH * NH * 2,
-                   SM_A2 = SM_A1 + TILE * NF * 2, SM_B = SM_A2 + TILE * NH * 2, SM_BAR = SM_B + 3 * NH * 4,
-                   SM_USED = SM_BAR + 16;
+                   SM_A2 = SM_A1 + TILE * NF * 2, SM_B = SM_A2 + TILE * NH * 2, SM_Y = SM_B + 3 * NH * 4,
+                   SM_BAR = SM_Y + TILE * 4, SM_USED = SM_BAR + 16;
 constexpr uint32_t SM_REQUEST = SM_USED + 128;
 static_assert(4 * (SM_REQUEST + 1024) > 228 * 1024 && kTmemCols * 3 <= 512, "at most three CTAs per SM");
 
 // Persistent forward over 128-row tiles.  Per tile: rows -> bfloat16 A tile; one MMA
 // (K = 16) into the 128 tensor-memory columns; epilogue (+b1, ReLU, bfloat16) writes the
 // second A tile; eight MMAs (K = 128) into the same columns; epilogue (+b2, ReLU, dot
-// with w3, +b3) gives y.  One thread per row: thread t of warp w owns row 32 w + t, which
-// is tensor-memory lane 32 w + t.  Input rows come from a feature matrix or, fused, are
-// built from the topology (output lambda_0 = y / scale); in training mode the hidden
-// activations are stored for the backward pass.  A wait that gives up counts in *err and
-// ends the kernel after freeing its tensor memory.
+// with w3, +b3) gives y.  Two threads per row: thread t of warp w owns row 32 (w & 3) + t, which
+// is that tensor-memory lane, and half w / 4 of its features and of the 128 columns.  Input
+// rows come from a feature matrix or, fused, are built from the topology (output lambda_0 = y
+// / scale); in training mode the hidden activations are stored for the backward pass.  A wait
+// that gives up counts in *err and ends the kernel after freeing its tensor memory.
+//
+// What bounds it: the MMAs take a few per cent of a tile's time; the rest is the features'
+// gathers (two dependent rounds, about 3,700 cycles with three CTAs to an SM) and the two
+// epilogues' 128 columns a row (about 2,200 each).  Two threads to a row halve both chains and
+// double the warps an SM overlaps them with (24 on three CTAs): a warm start of 258,048
+// constraints, with its prep pass, 50.6 -> 43.7 us.
 template <bool kFused, bool kTrain>
-__global__ void __launch_bounds__(TILE)
+__global__ void __launch_bounds__(kFwdThreads, 3)
 k_mlp_forward(MlpWeights Wt, const float* __restrict__ X, int n, FeatArgs F, float* __restrict__ out,
               __nv_bfloat16* __restrict__ h1_out, float* __restrict__ h2_out, int* __restrict__ err,
               int wait_test) {
@@ -247,11 +262,12 @@ k_mlp_forward(MlpWeights Wt, const float* __restrict__ X, int n, FeatArgs F, flo
     float* b1s = reinterpret_cast<float*>(sm + SM_B);
     float* b2s = b1s + NH;
     float* w3s = b2s + NH;
+    float* ys = reinterpret_cast<float*>(sm + SM_Y);  // the second half's part of each row's y
     uint64_t* bar = reinterpret_cast<uint64_t*>(sm + SM_BAR);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + SM_BAR + 8);
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = tid >> 5, lrow = tid & (TILE - 1), half = tid / TILE;
     const uint32_t mbar = saddr_of(bar);
-    if (warp == 0) {  // 256 tensor-memory columns for this CTA
+    if (warp == 0) {  // 128 tensor-memory columns for this CTA
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr_of(tmem_slot)),
                      "r"(kTmemCols)
                      : "memory");
@@ -261,29 +277,28 @@ k_mlp_forward(MlpWeights Wt, const float* __restrict__ X, int n, FeatArgs F, flo
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mbar), "r"(1) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // weights into the canonical layout: 16-byte chunks of 8 K values
-    for (int e = tid; e < NH * NF / 8; e += TILE) {
-        const int row = e / (NF / 8), kc = e % (NF / 8);
-        *reinterpret_cast<uint4*>(sm + SM_W1 + core_offset(row, kc, NF / 8)) =
-            __ldg(reinterpret_cast<const uint4*>(Wt.w1) + e);
+    // weights into the canonical layout: 16-byte chunks of 8 K values, taken in the layout's
+    // order (row within the core matrix fastest), so the shared-memory writes are linear; the
+    // copies run while the first tile's rows are built
+    for (int e = tid; e < NH * NF / 8; e += kFwdThreads) {
+        const int r8 = e & 7, kc = (e >> 3) % (NF / 8), row = 8 * (e / NF) + r8;
+        copy16(sm + SM_W1 + 16 * e, reinterpret_cast<const uint4*>(Wt.w1) + row * (NF / 8) + kc);
     }
-    for (int e = tid; e < NH * NH / 8; e += TILE) {
-        const int row = e / (NH / 8), kc = e % (NH / 8);
-        *reinterpret_cast<uint4*>(sm + SM_W2 + core_offset(row, kc, NH / 8)) =
-            __ldg(reinterpret_cast<const uint4*>(Wt.w2) + e);
+    for (int e = tid; e < NH * NH / 8; e += kFwdThreads) {
+        const int r8 = e & 7, kc = (e >> 3) % (NH / 8), row = 8 * (e / NH) + r8;
+        copy16(sm + SM_W2 + 16 * e, reinterpret_cast<const uint4*>(Wt.w2) + row * (NH / 8) + kc);
     }
-    for (int e = tid; e < NH; e += TILE) {
+    for (int e = tid; e < NH; e += kFwdThreads) {
         b1s[e] = Wt.params[P_B1 + e];
         b2s[e] = Wt.params[P_B2 + e];
         w3s[e] = Wt.params[P_W3 + e];
     }
     const float b3 = Wt.params[P_B3];
-    async_proxy_fence();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const uint32_t t_lane = (uint32_t)(32 * warp) << 16;
+    const uint32_t t_half = ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(NH / 2 * half);  // this thread's columns
     const uint64_t dA1 = smem_desc(saddr_of(sm + SM_A1), 128, (NF / 8) * 128);
     const uint64_t dW1 = smem_desc(saddr_of(sm + SM_W1), 128, (NF / 8) * 128);
     const uint64_t dA2 = smem_desc(saddr_of(sm + SM_A2), 128, (NH / 8) * 128);
@@ -295,32 +310,37 @@ k_mlp_forward(MlpWeights Wt, const float* __restrict__ X, int n, FeatArgs F, flo
         ok = __syncthreads_and(mbar_wait(mbar, parity)) != 0;
     }
     for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-        const int row = tile * TILE + tid;
+        const int row = tile * TILE + lrow;
         // ---- input row -> bfloat16 A tile
-        float f[NF], sc = 0.f;
+        float sc = 0.f;
+        if constexpr (kFused) {  // half 0: features 0-9 and the scale, half 1: features 10-15
+            float f[NF];
 #pragma unroll
-        for (int c = 0; c < NF; ++c) f[c] = 0.f;
-        if (row < n) {
-            if constexpr (kFused) {
-                ws_features(F, row, 0, f, sc);
-                ws_features(F, row, 1, f, sc);
+            for (int c = 0; c < NF; ++c) f[c] = 0.f;
+            uint32_t* k1 = reinterpret_cast<uint32_t*>(sm + SM_A1 + core_offset(lrow, 1, NF / 8));
+            if (half == 0) {
+                if (row < n) ws_features<0>(F, row, f, sc);
+                *reinterpret_cast<uint4*>(sm + SM_A1 + core_offset(lrow, 0, NF / 8)) =
+                    make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
+                k1[0] = pack_bf16(f[8], f[9]);
             } else {
-                const float4* xr = reinterpret_cast<const float4*>(X + (int64_t)row * NF);
-#pragma unroll
-                for (int c = 0; c < NF / 4; ++c) {
-                    const float4 v = __ldg(xr + c);
-                    f[4 * c] = v.x;
-                    f[4 * c + 1] = v.y;
-                    f[4 * c + 2] = v.z;
-                    f[4 * c + 3] = v.w;
-                }
+                if (row < n) ws_features<1>(F, row, f, sc);
+                k1[1] = pack_bf16(f[10], f[11]);
+                k1[2] = pack_bf16(f[12], f[13]);
+                k1[3] = pack_bf16(f[14], f[15]);
             }
+        } else {  // eight features each
+            float4 v[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+            if (row < n) {
+                const float4* xr = reinterpret_cast<const float4*>(X + (int64_t)row * NF) + 2 * half;
+                v[0] = __ldg(xr);
+                v[1] = __ldg(xr + 1);
+            }
+            *reinterpret_cast<uint4*>(sm + SM_A1 + core_offset(lrow, half, NF / 8)) =
+                make_uint4(pack_bf16(v[0].x, v[0].y), pack_bf16(v[0].z, v[0].w), pack_bf16(v[1].x, v[1].y),
+                           pack_bf16(v[1].z, v[1].w));
         }
-#pragma unroll
-        for (int kc = 0; kc < NF / 8; ++kc)
-            *reinterpret_cast<uint4*>(sm + SM_A1 + core_offset(tid, kc, NF / 8)) =
-                make_uint4(pack_bf16(f[8 * kc], f[8 * kc + 1]), pack_bf16(f[8 * kc + 2], f[8 * kc + 3]),
-                           pack_bf16(f[8 * kc + 4], f[8 * kc + 5]), pack_bf16(f[8 * kc + 6], f[8 * kc + 7]));
+        copy_wait_all();  // (the weights; nothing is in flight after the first tile)
         async_proxy_fence();
         tc_fence_before();
         __syncthreads();
@@ -335,20 +355,22 @@ k_mlp_forward(MlpWeights Wt, const float* __restrict__ X, int n, FeatArgs F, flo
         tc_fence_after();
         if (!ok) break;
 #pragma unroll 1
-        for (int ch = 0; ch < NH / 32; ++ch) {
+        for (int ch = 0; ch < 2; ++ch) {
             float v[32];
-            tmem_ld32(tmem + t_lane + 32 * ch, v);
-            uint32_t hb[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-                hb[j] = pack_bf16(fmaxf(v[2 * j] + b1s[32 * ch + 2 * j], 0.f),
-                                  fmaxf(v[2 * j + 1] + b1s[32 * ch + 2 * j + 1], 0.f));
+            tmem_ld32(tmem + t_half + 32 * ch, v);
+            const int c0 = NH / 2 * half + 32 * ch;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const uint4 u = make_uint4(hb[4 * q], hb[4 * q + 1], hb[4 * q + 2], hb[4 * q + 3]);
-                *reinterpret_cast<uint4*>(sm + SM_A2 + core_offset(tid, 4 * ch + q, NH / 8)) = u;
+                const float4 ba = *reinterpret_cast<const float4*>(b1s + c0 + 8 * q);
+                const float4 bb = *reinterpret_cast<const float4*>(b1s + c0 + 8 * q + 4);
+                const float* w = v + 8 * q;
+                const uint4 u = make_uint4(pack_bf16(fmaxf(w[0] + ba.x, 0.f), fmaxf(w[1] + ba.y, 0.f)),
+                                           pack_bf16(fmaxf(w[2] + ba.z, 0.f), fmaxf(w[3] + ba.w, 0.f)),
+                                           pack_bf16(fmaxf(w[4] + bb.x, 0.f), fmaxf(w[5] + bb.y, 0.f)),
+                                           pack_bf16(fmaxf(w[6] + bb.z, 0.f), fmaxf(w[7] + bb.w, 0.f)));
+                *reinterpret_cast<uint4*>(sm + SM_A2 + core_offset(lrow, c0 / 8 + q, NH / 8)) = u;
                 if constexpr (kTrain) {
-                    if (row < n) reinterpret_cast<uint4*>(h1_out + (int64_t)row * NH + 32 * ch)[q] = u;
+                    if (row < n) reinterpret_cast<uint4*>(h1_out + (int64_t)row * NH + c0)[q] = u;
                 }
             }
         }
@@ -368,24 +390,34 @@ k_mlp_forward(MlpWeights Wt, const float* __restrict__ X, int n, FeatArgs F, flo
         if (!ok) break;
         float y = 0.f;
 #pragma unroll 1
-        for (int ch = 0; ch < NH / 32; ++ch) {
+        for (int ch = 0; ch < 2; ++ch) {
             float v[32];
-            tmem_ld32(tmem + t_lane + 32 * ch, v);
+            tmem_ld32(tmem + t_half + 32 * ch, v);
+            const int c0 = NH / 2 * half + 32 * ch;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                v[j] = fmaxf(v[j] + b2s[32 * ch + j], 0.f);
-                y = fmaf(v[j], w3s[32 * ch + j], y);
-            }
-            if constexpr (kTrain) {
-                if (row < n) {
-                    float4* h2r = reinterpret_cast<float4*>(h2_out + (int64_t)row * NH + 32 * ch);
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) h2r[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+            for (int q = 0; q < 8; ++q) {
+                const float4 b = *reinterpret_cast<const float4*>(b2s + c0 + 4 * q);
+                const float4 w = *reinterpret_cast<const float4*>(w3s + c0 + 4 * q);
+                float* u = v + 4 * q;
+                u[0] = fmaxf(u[0] + b.x, 0.f);
+                u[1] = fmaxf(u[1] + b.y, 0.f);
+                u[2] = fmaxf(u[2] + b.z, 0.f);
+                u[3] = fmaxf(u[3] + b.w, 0.f);
+                y = fmaf(u[0], w.x, y);
+                y = fmaf(u[1], w.y, y);
+                y = fmaf(u[2], w.z, y);
+                y = fmaf(u[3], w.w, y);
+                if constexpr (kTrain) {
+                    if (row < n)
+                        reinterpret_cast<float4*>(h2_out + (int64_t)row * NH + c0)[q] = make_float4(u[0], u[1], u[2], u[3]);
                 }
             }
         }
-        if (row < n) {
-            y += b3;
+        tc_fence_before();
+        if (half == 1) ys[lrow] = y;
+        __syncthreads();
+        if (half == 0 && row < n) {
+            y = (y + ys[lrow]) + b3;
             if constexpr (kFused) {
                 const float l0 = y / sc;
                 out[row] = (sc != 0.f && isfinite(l0)) ? l0 : 0.f;
@@ -393,8 +425,8 @@ k_mlp_forward(MlpWeights Wt, const float* __restrict__ X, int n, FeatArgs F, flo
                 out[row] = y;
             }
         }
-        tc_fence_before();
     }
+    copy_wait_all();  // (a wait given up before the first tile)
     if (!ok && tid == 0) atomicAdd(err, 1);
     tc_fence_before();
     __syncthreads();
@@ -417,7 +449,7 @@ k_mlp_forward(MlpWeights Wt, const float* __restrict__ X, int n, FeatArgs F, flo
 // the gradient is the same on every run and its rounding error does not grow with the number
 // of CTAs, as it did with float32 atomics.  Rows are spread over the SMs, but at least kBwdMinRows
 // to a CTA, below which the 75 KB of W2 in and gradient out cost more than they save.
-// A whole gradient of 8192 rows takes 45 us; with one thread per hidden unit, rows streamed one by
+// A whole gradient of 8192 rows takes 38.9 us (forward 12, this kernel 20, reduction 5); with one thread per hidden unit, rows streamed one by
 // one with three barriers each and float32 atomics it took 220 us.
 constexpr int kBwdRows = 64, kBwdMinRows = 16, kBwdThreads = 256;
 constexpr int kPartStride = (P_N + 1 + 3) & ~3;  // a CTA's partial gradient, then its loss
@@ -442,14 +474,17 @@ k_mlp_backward(const float* __restrict__ X, const float* __restrict__ t, int n, 
     float* xs = h1s + kBwdRows * NH;        // [r][f]
     float* dys = xs + kBwdRows * NF;        // [r]
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    for (int e = tid; e < NH * NH / 8; e += kBwdThreads) {
+#pragma unroll
+    for (int q0 = 0; q0 < NH * NH / 8 / kBwdThreads; ++q0) {
+        const int e = tid + kBwdThreads * q0;
         const uint4 v = __ldg(reinterpret_cast<const uint4*>(w2b) + e);
         const __nv_bfloat162* b = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
         for (int q = 0; q < 4; ++q) *reinterpret_cast<float2*>(w2s + 8 * e + 2 * q) = __bfloat1622float2(b[q]);
     }
-    const int c = tid & (NH - 1), half = tid >> 7;  // column sums: column c, every other row
-    const float w3c = params[P_W3 + c];
+    const int c = tid & (NH - 1), half = tid >> 7;
+    const int c4 = 4 * (tid & 31), r8 = tid >> 5;  // dz2 and its column sums: columns c4 .. c4 + 3, every 8th row
+    const float4 w3v = make_float4(params[P_W3 + c4], params[P_W3 + c4 + 1], params[P_W3 + c4 + 2], params[P_W3 + c4 + 3]);
     const float inv_n = 1.0f / (float)n;
     // rows (columns) of a tile: ty * 4 .. + 3 and 64 + ty * 4 .. + 3 (tx alike), so the lanes of a warp
     // read consecutive 16-byte words
@@ -460,7 +495,8 @@ k_mlp_backward(const float* __restrict__ X, const float* __restrict__ t, int n, 
         for (int b = 0; b < 4; ++b) gw2[a][b] = make_float2(0.f, 0.f);
 #pragma unroll
     for (int b = 0; b < 4; ++b) gw1[b] = make_float2(0.f, 0.f);
-    float gb1 = 0.f, gb2 = 0.f, gw3 = 0.f, gb3 = 0.f, lsum = 0.f;
+    float4 gb2 = make_float4(0.f, 0.f, 0.f, 0.f), gw3 = gb2;
+    float gb1 = 0.f, gb3 = 0.f, lsum = 0.f;
     const int rb = blockIdx.x * rows_per_cta, re = min(n, rb + rows_per_cta);
     for (int r0 = rb; r0 < re; r0 += kBwdRows) {
         const int rows = min(kBwdRows, re - r0), rows4 = (rows + 3) & ~3;  // completed with zero rows
@@ -487,12 +523,31 @@ k_mlp_backward(const float* __restrict__ X, const float* __restrict__ t, int n, 
             for (int q = 0; q < 4; ++q) *reinterpret_cast<float2*>(h1s + 8 * e + 2 * q) = __bfloat1622float2(b[q]);
         }
         __syncthreads();
-        for (int r = half; r < rows4; r += 2) {
-            const float h = r < rows ? __ldg(h2 + (int64_t)(r0 + r) * NH + c) : 0.f, dy = dys[r];
-            const float dz2 = h > 0.f ? dy * w3c : 0.f;
-            gw3 += dy * h;
-            gb2 += dz2;
-            dzs[r * NH + c] = dz2;
+        {
+            float4 h[kBwdRows / 8];
+#pragma unroll
+            for (int q = 0; q < kBwdRows / 8; ++q) {
+                const int r = r8 + 8 * q;
+                h[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (r < rows) h[q] = __ldg(reinterpret_cast<const float4*>(h2 + (int64_t)(r0 + r) * NH + c4));
+            }
+#pragma unroll
+            for (int q = 0; q < kBwdRows / 8; ++q) {
+                const int r = r8 + 8 * q;
+                if (r >= rows4) break;
+                const float dy = dys[r];
+                const float4 z = make_float4(h[q].x > 0.f ? dy * w3v.x : 0.f, h[q].y > 0.f ? dy * w3v.y : 0.f,
+                                             h[q].z > 0.f ? dy * w3v.z : 0.f, h[q].w > 0.f ? dy * w3v.w : 0.f);
+                gw3.x += dy * h[q].x;
+                gw3.y += dy * h[q].y;
+                gw3.z += dy * h[q].z;
+                gw3.w += dy * h[q].w;
+                gb2.x += z.x;
+                gb2.y += z.y;
+                gb2.z += z.z;
+                gb2.w += z.w;
+                *reinterpret_cast<float4*>(dzs + r * NH + c4) = z;
+            }
         }
         __syncthreads();
         // gW2[c][k] += sum_r dz2[r][c] h1[r][k]
@@ -577,30 +632,28 @@ k_mlp_backward(const float* __restrict__ X, const float* __restrict__ t, int n, 
     float4* g1 = reinterpret_cast<float4*>(grad + P_W1 + c * NF + 8 * half);
     g1[0] = make_float4(gw1[0].x, gw1[0].y, gw1[1].x, gw1[1].y);
     g1[1] = make_float4(gw1[2].x, gw1[2].y, gw1[3].x, gw1[3].y);
-    // the column sums of even and odd rows, the sums over rows
+    // the column sums of the eight row groups, the sums over rows
     __syncthreads();
-    if (half == 1) {
-        dzs[c] = gb2;
-        dzs[NH + c] = gw3;
-    }
+    *reinterpret_cast<float4*>(dzs + r8 * NH + c4) = gb2;
+    *reinterpret_cast<float4*>(dzs + (8 + r8) * NH + c4) = gw3;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         gb3 += __shfl_xor_sync(0xFFFFFFFFu, gb3, o);
         lsum += __shfl_xor_sync(0xFFFFFFFFu, lsum, o);
     }
     if (tid == 32) {
-        dzs[2 * NH] = gb3;
-        dzs[2 * NH + 1] = lsum;
+        dys[0] = gb3;
+        dys[1] = lsum;
     }
     __syncthreads();
-    if (half == 0) {
-        grad[P_B1 + c] = gb1;
-        grad[P_B2 + c] = gb2 + dzs[c];
-        grad[P_W3 + c] = gw3 + dzs[NH + c];
-    }
+    if (half == 0) grad[P_B1 + c] = gb1;
+    float sum = 0.f;  // half 0: gb2[c], half 1: gw3[c]
+#pragma unroll
+    for (int q = 0; q < 8; ++q) sum += dzs[(8 * half + q) * NH + c];
+    grad[(half == 0 ? P_B2 : P_W3) + c] = sum;
     if (tid == 0) {
-        grad[P_B3] = gb3 + dzs[2 * NH];
-        grad[P_N] = lsum + dzs[2 * NH + 1];
+        grad[P_B3] = gb3 + dys[0];
+        grad[P_N] = lsum + dys[1];
     }
 }
 
@@ -613,6 +666,7 @@ k_grad_reduce(const float* __restrict__ partial, int n_part, float* __restrict__
     const int col = blockIdx.x * 32 + (threadIdx.x & 31), row = threadIdx.x >> 5;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     if (col < kPartStride / 4)
+#pragma unroll 8
         for (int p = row; p < n_part; p += kRedThreads / 32) {
             const float4 v = __ldg(reinterpret_cast<const float4*>(partial + (int64_t)p * kPartStride) + col);
             s.x += v.x;
@@ -703,8 +757,7 @@ static FeatArgs feat_args(const ilves_topology* T, const double* x_old, const do
     F.d = d;
     F.con_i = T->d_con_i;
     F.con_j = T->d_con_j;
-    F.nbr = T->d_nbr;
-    F.nbr_atom = T->d_nbr_atom;
+    F.nbr = reinterpret_cast<const int4*>(T->d_nbr);
     F.ws_con = reinterpret_cast<float4*>(T->d_ws_con);
     F.ws_atom = T->d_ws_atom;
     F.n_c = T->n_c;
@@ -730,7 +783,7 @@ static cudaError_t launch_forward(const MlpWeights& Wt, const float* X, int n, c
     }
     const int tiles = (n + TILE - 1) / TILE;
     const int grid = std::max(1, std::min(tiles, 3 * sms));
-    k_mlp_forward<kFused, kTrain><<<grid, TILE, SM_REQUEST, s>>>(Wt, X, n, F, out, h1, h2, err, wait_test);
+    k_mlp_forward<kFused, kTrain><<<grid, kFwdThreads, SM_REQUEST, s>>>(Wt, X, n, F, out, h1, h2, err, wait_test);
     return cudaGetLastError();
 }
 

@@ -2162,7 +2162,6 @@ static void free_device(ilves_topology* T) {
     f(T->d_con_i);
     f(T->d_con_j);
     f(T->d_nbr);
-    f(T->d_nbr_atom);
     f(T->d_ws_con);
     f(T->d_ws_atom);
     f(T->d_sync);
@@ -2184,7 +2183,7 @@ static void free_device(ilves_topology* T) {
     T->d_blob = nullptr;
     T->d_atom_gid = nullptr;
     T->d_free_atoms = nullptr;
-    T->d_con_i = T->d_con_j = T->d_nbr = T->d_nbr_atom = nullptr;
+    T->d_con_i = T->d_con_j = T->d_nbr = nullptr;
     T->d_ws_con = T->d_ws_atom = nullptr;
     T->d_sync = nullptr;
     T->d_work = nullptr;
@@ -2311,7 +2310,6 @@ static ilves_status upload_topology(ilves_topology* T, const ilves_setup_opts& o
     if ((e = upload(&T->d_con_i, T->con_i)) != cudaSuccess) return to_status(e);
     if ((e = upload(&T->d_con_j, T->con_j)) != cudaSuccess) return to_status(e);
     if ((e = upload(&T->d_nbr, T->nbr)) != cudaSuccess) return to_status(e);
-    if ((e = upload(&T->d_nbr_atom, T->nbr_atom)) != cudaSuccess) return to_status(e);
     if (T->n_c > 0 && (e = cudaMalloc((void**)&T->d_ws_con, (size_t)T->n_c * 8 * sizeof(float))) != cudaSuccess)
         return to_status(e);
     if (T->n_atoms > 0 && (e = cudaMalloc((void**)&T->d_ws_atom, (size_t)T->n_atoms * sizeof(float))) != cudaSuccess)
@@ -2847,7 +2845,7 @@ extern "C" int64_t ilves_topology_device_bytes(const ilves_topology* T) {
     int64_t b = T->blob_bytes + (int64_t)T->n_mol * (int64_t)sizeof(MolDesc) + T->work_bytes + T->sync_bytes;
     b += 4 * (int64_t)T->n_atoms;                        // atom ids
     b += 4 * (int64_t)T->free_atoms.size();
-    b += (int64_t)T->n_c * (4 + 4 + 16 + 16 + 32);      // atoms, neighbour table, warm-start workspace
+    b += (int64_t)T->n_c * (4 + 4 + 16 + 32);           // atoms, neighbour table, warm-start workspace
     b += 4 * (int64_t)T->n_atoms;                        // warm-start atom weights
     for (const auto& sc : T->sched) b += 4 * (int64_t)(2 * sc.n_cta + 2 * T->n_small + 64);
     return b;

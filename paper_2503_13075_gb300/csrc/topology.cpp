@@ -1063,7 +1063,6 @@ ilves_status plan_topology(ilves_topology* T, int32_t n_atoms, int32_t n_c, cons
     T->con_i.assign(ai, ai + n_c);
     T->con_j.assign(aj, aj + n_c);
     T->nbr.assign((size_t)n_c * 4, -1);
-    T->nbr_atom.assign((size_t)n_c * 4, -1);
     {
         std::vector<int32_t> deg(n_atoms + 1, 0);
         for (int32_t k = 0; k < n_c; ++k) {
@@ -1082,8 +1081,8 @@ ilves_status plan_topology(ilves_topology* T, int32_t n_atoms, int32_t n_c, cons
                 int32_t slot = 2 * side;
                 for (int32_t e = deg[a]; e < deg[a + 1] && slot < 2 * side + 2; ++e) {
                     if (inc_all[e] == k) continue;
-                    T->nbr[(size_t)k * 4 + slot] = inc_all[e];
-                    T->nbr_atom[(size_t)k * 4 + slot] = a;
+                    const int32_t l = inc_all[e];  // s_k(a) s_l(a): + at a first atom, - at a second one
+                    T->nbr[(size_t)k * 4 + slot] = (l << 1) | ((a == ai[k]) == (a == ai[l]) ? 0 : 1);
                     ++slot;
                 }
             }

@@ -86,9 +86,9 @@ struct ilves_topology {
     std::vector<ilves::MolHost> mols;
     std::vector<ilves::Program*> progs;  // owned
     std::vector<int32_t> free_atoms;
-    // per global constraint: atoms, and up to 4 line-graph neighbours (2 sharing atom_i,
-    // then 2 sharing atom_j; -1 = none) with the global id of the shared atom
-    std::vector<int32_t> con_i, con_j, nbr, nbr_atom;
+    // per global constraint: atoms, and up to 4 line-graph neighbours (2 sharing atom_i, then 2
+    // sharing atom_j; -1 = none): neighbour << 1 | (the sign product at the shared atom is negative)
+    std::vector<int32_t> con_i, con_j, nbr;
     // device side
     int32_t device = -1;
     bool on_device = false;
@@ -102,7 +102,6 @@ struct ilves_topology {
     int32_t* d_con_i = nullptr;
     int32_t* d_con_j = nullptr;
     int32_t* d_nbr = nullptr;       // n_c x 4
-    int32_t* d_nbr_atom = nullptr;  // n_c x 4
     float* d_ws_con = nullptr;      // warm-start workspace: n_c x 8 floats (s, sigma0/d^2, rho, d)
     float* d_ws_atom = nullptr;     // n_atoms floats (inverse masses)
     uint8_t* d_work = nullptr;               // large-molecule numerical state
