@@ -1262,7 +1262,7 @@ __device__ __forceinline__ bool grid_sync(unsigned long long* ctr, unsigned n_bl
 // Shared memory of the separator phase: rows (V4) and right-hand sides of the
 // separators, values of the separator tasks; the separators' reference rows and the
 // tasks' assembly coefficients; with stage_ct, a copy of the parts' contributions (4 per
-// task); the separator program.  Used when it fits kPartedSmemMax.
+// task); the separator program.  Used when it fits parted_smem_limit.
 template <class Mode>
 __host__ __device__ inline uint32_t sep_smem_bytes(int nsep, int n_sept, int sprog_bytes, bool stage_ct) {
     using LP = typename Mode::LP;
@@ -1289,7 +1289,15 @@ __host__ __device__ inline uint32_t part_prog_smem_bytes(int na, int np, int nt,
     return part_smem_bytes<Mode>(na, np, nt) + align16((uint32_t)sizeof(V4) * np) +
            align16((uint32_t)sizeof(LP) * na) + (uint32_t)prog_max;
 }
-constexpr uint32_t kPartedSmemMax = 72 * 1024;  // three CTAs per SM still fit
+// Dynamic shared memory a CTA of a partitioned launch may take: an SM's, over the CTAs each SM has
+// to hold for all n_cta of them to be resident at once (at most three).  Parts of 256
+// constraints need 75 KB in float64 with their programs: with 72 KB for every launch a system
+// of 20,000 atoms (91 parts on 152 SMs) ran them from global memory, 501 us against 327 us.
+constexpr uint32_t kPartedSmemMax = 231424;
+inline uint32_t parted_smem_limit(int n_cta, int n_sm) {
+    const int per_sm = (n_cta + n_sm - 1) / std::max(1, n_sm);
+    return per_sm <= 1 ? kPartedSmemMax : per_sm == 2 ? 115712u : 72u * 1024u;
+}
 
 // Dynamic shared memory of a partitioned launch: the separator block (0 = it stays in
 // global memory) of CTA sep_cta, and the part copies (0 = off; on only with one part per
@@ -2430,14 +2438,15 @@ static ilves_status launch_all(ilves_topology* T, const SolveArgs& A, cudaStream
                 // shared memory: the separator block if it fits, then the parts' copies if
                 // every part gets a CTA of its own at that size
                 // (with a staged copy of the contributions if that fits too)
+                const uint32_t limit = parted_smem_limit(n_parts + 1, T->n_sm);
                 uint32_t sep_b = 0, sep_ct = 0;
                 if (MH.sprog_bytes > 0) {
                     const uint32_t with_ct = sep_smem_bytes<Mode>(MH.n_sep, MH.n_sept, MH.sprog_bytes, true);
                     const uint32_t without = sep_smem_bytes<Mode>(MH.n_sep, MH.n_sept, MH.sprog_bytes, false);
-                    if (with_ct <= kPartedSmemMax) {
+                    if (with_ct <= limit) {
                         sep_b = with_ct;
                         sep_ct = 1;
-                    } else if (without <= kPartedSmemMax) {
+                    } else if (without <= limit) {
                         sep_b = without;
                     }
                 }
@@ -2470,7 +2479,7 @@ static ilves_status launch_all(ilves_topology* T, const SolveArgs& A, cudaStream
                     if (c.prog && !pp) continue;
                     const size_t d = c.sep_cta == 0 ? align16(c.sep_bytes) + c.part_bytes
                                                      : std::max<size_t>(c.sep_bytes, c.part_bytes);
-                    if (d > kPartedSmemMax) continue;
+                    if (d > limit) continue;
                     int per_sm = 0;
                     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_parted<Mode>,
                                                                            T->parted_threads, d)) != cudaSuccess)

@@ -1111,6 +1111,17 @@ ilves_status plan_topology(ilves_topology* T, int32_t n_atoms, int32_t n_c, cons
         const int64_t wide_teams = (int64_t)kMaxSlotsPerCta * (T->n_sm > 0 ? T->n_sm : 152);
         if (n_batched > wide_teams && small * 10 >= batched * 9) narrow = kDefaultNarrowAtoms;
     }
+    // Automatic partition threshold: 4096 constraints, or kLonePartitionMin for a topology's only
+    // molecule that is too large for the batched kernel.  Its parts run on several SMs where one
+    // CTA has one SM's float64 pipe (a tree of 1400 atoms, mixed / float64: 119 / 242 us against
+    // 189 / 358; 4000 atoms: 154 / 326 against 425 / 767; even at 900 constraints).  Several such
+    // molecules share one launch of a CTA each, while partitioned solves run one after another.
+    constexpr int32_t kLonePartitionMin = 1000;
+    int32_t n_big = 0;
+    for (const MolHost& M : T->mols)
+        if ((int32_t)M.cons.size() > warp_limit || (int32_t)M.cons.size() >= (int32_t)kCompactMaxConstraints ||
+            (int32_t)M.atoms.size() > (int32_t)PairWord::kMaxAtom)
+            ++n_big;
     std::vector<std::vector<int32_t>> inc, adj;
     for (int32_t m = 0; m < n_mol; ++m) {
         MolHost& M = T->mols[m];
@@ -1176,7 +1187,7 @@ ilves_status plan_topology(ilves_topology* T, int32_t n_atoms, int32_t n_c, cons
             M.n_dom = 0;
             for (int32_t& v : M.dom_smem) v = 0;
         }
-        if (nc >= part_min) {
+        if (nc >= part_min || (o.partition_min_constraints <= 0 && n_big == 1 && M.large && nc >= kLonePartitionMin)) {
             // partitioned: parts of ~part_size constraints eliminated first, separators last
             M.large = M.parted = true;
             // automatic part size: about 256 constraints, but never more parts (plus the
