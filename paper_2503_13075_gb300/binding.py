@@ -141,6 +141,28 @@ def _check(code, where):
         raise IlvesError(code, where)
 
 
+_torch_module = None
+
+
+def _torch():
+    global _torch_module
+    if _torch_module is None:
+        import torch
+
+        _torch_module = torch
+    return _torch_module
+
+
+def _placed(t, dev):
+    """On the solve's device, or in page-locked host memory."""
+    return t.device == dev or (t.device.type == "cpu" and t.is_pinned())
+
+
+def _refuse(name, shape):
+    raise ValueError(f"{name} must be a contiguous float64 tensor of shape {shape}, "
+                     "on the CUDA device or in pinned host memory")
+
+
 class Topology:
     """A constraint topology set up once and solved many times (``ilves_setup_topology``)."""
 
@@ -337,45 +359,46 @@ class Topology:
         kernels read or write in place; outputs not given are allocated like ``x_unc``.
         ``start="diag"`` computes the diagonal starting multipliers inside the solve
         (``ILVES_START_DIAG``; lambda0 must then be None)."""
-        import torch
-
+        torch = _torch()
         if self.plan_only:
             raise RuntimeError("topology was planned on the host only")
-        given = [t for t in (x_old, x_unc, inv_mass, d, lambda0, x_out, lambda_out, iterations_out, status_out)
-                 if t is not None]
-        dev = next((t.device for t in given if t.is_cuda), None)
+        dev = x_old.device if x_old.is_cuda else next(
+            (t.device for t in (x_unc, inv_mass, d, lambda0, x_out, lambda_out, iterations_out, status_out)
+             if t is not None and t.is_cuda), None)
         if dev is None:
             dev = torch.device("cuda", self._device_index if self._device_index is not None
                                else torch.cuda.current_device())
-
-        def placed(t):  # on the solve's device, or page-locked host memory
-            return t.device == dev or (t.device.type == "cpu" and t.is_pinned())
-
-        for name, t, shape in (("x_old", x_old, (self.n_atoms, 3)), ("x_unc", x_unc, (self.n_atoms, 3)),
-                               ("inv_mass", inv_mass, (self.n_atoms,)), ("d", d, (self.n_constraints,))):
-            if t.dtype != torch.float64 or tuple(t.shape) != shape or not t.is_contiguous() or not placed(t):
-                raise ValueError(f"{name} must be a contiguous float64 tensor of shape {shape}, "
-                                 "on the CUDA device or in pinned host memory")
-        if lambda0 is not None and (lambda0.dtype != torch.float32 or lambda0.numel() != self.n_constraints
-                                    or not lambda0.is_contiguous() or not placed(lambda0)):
+        f64 = torch.float64
+        n_atoms, n_con, n_mol = self.n_atoms, self.n_constraints, self.n_molecules
+        # a call of a few launches is bound by this function, so the checks are written out and
+        # the tensors it makes itself are not checked again
+        if not (x_old.dtype == f64 and x_old.shape == (n_atoms, 3) and x_old.is_contiguous() and _placed(x_old, dev)):
+            _refuse("x_old", (n_atoms, 3))
+        if not (x_unc.dtype == f64 and x_unc.shape == (n_atoms, 3) and x_unc.is_contiguous() and _placed(x_unc, dev)):
+            _refuse("x_unc", (n_atoms, 3))
+        if not (inv_mass.dtype == f64 and inv_mass.shape == (n_atoms,) and inv_mass.is_contiguous()
+                and _placed(inv_mass, dev)):
+            _refuse("inv_mass", (n_atoms,))
+        if not (d.dtype == f64 and d.shape == (n_con,) and d.is_contiguous() and _placed(d, dev)):
+            _refuse("d", (n_con,))
+        if lambda0 is not None and (lambda0.dtype != torch.float32 or lambda0.numel() != n_con
+                                    or not lambda0.is_contiguous() or not _placed(lambda0, dev)):
             raise ValueError("lambda0 must be a contiguous float32 tensor of n_constraints entries")
-        host = x_unc.device.type == "cpu"
-
-        def alloc(n, dtype):
-            return torch.empty(n, dtype=dtype, pin_memory=True) if host else torch.empty(n, dtype=dtype, device=dev)
-
-        x_out = alloc((self.n_atoms, 3), torch.float64) if x_out is None else x_out
-        lambda_out = alloc(self.n_constraints, torch.float64) if lambda_out is None else lambda_out
-        iterations_out = alloc(self.n_molecules, torch.int32) if iterations_out is None else iterations_out
-        status_out = alloc(self.n_molecules, torch.int32) if status_out is None else status_out
-        for name, t, dtype, n in (("x_out", x_out, torch.float64, 3 * self.n_atoms),
-                                  ("lambda_out", lambda_out, torch.float64, self.n_constraints),
-                                  ("iterations_out", iterations_out, torch.int32, self.n_molecules),
-                                  ("status_out", status_out, torch.int32, self.n_molecules)):
-            if t.dtype != dtype or t.numel() != n or not t.is_contiguous() or not placed(t):
+        place = {"pin_memory": True} if x_unc.device.type == "cpu" else {"device": dev}
+        for name, t, dtype, n in (("x_out", x_out, f64, 3 * n_atoms), ("lambda_out", lambda_out, f64, n_con),
+                                  ("iterations_out", iterations_out, torch.int32, n_mol),
+                                  ("status_out", status_out, torch.int32, n_mol)):
+            if t is not None and (t.dtype != dtype or t.numel() != n or not t.is_contiguous() or not _placed(t, dev)):
                 raise ValueError(f"{name} must be a contiguous {dtype} tensor of {n} entries, "
                                  "on the CUDA device or in pinned host memory")
-        s = torch.cuda.current_stream(dev).cuda_stream if stream is None else stream.cuda_stream
+        if x_out is None:
+            x_out = torch.empty((n_atoms, 3), dtype=f64, **place)
+        if lambda_out is None:
+            lambda_out = torch.empty(n_con, dtype=f64, **place)
+        if iterations_out is None:
+            iterations_out = torch.empty(n_mol, dtype=torch.int32, **place)
+        if status_out is None:
+            status_out = torch.empty(n_mol, dtype=torch.int32, **place)
         prec = PRECISIONS[precision] if isinstance(precision, str) else int(precision)
         if method == "chord":
             prec |= CHORD
@@ -387,10 +410,13 @@ class Topology:
             prec |= START_DIAG
         elif start is not None:
             raise ValueError("start must be None or 'diag'")
-        fn = getattr(lib(), _entry)
-        _check(fn(self._h, _ptr(x_old), _ptr(x_unc), _ptr(inv_mass), _ptr(d), float(tol), int(max_iter),
-                  prec, None if lambda0 is None else _ptr(lambda0), _ptr(x_out), _ptr(lambda_out),
-                  _ptr(iterations_out), _ptr(status_out), ctypes.c_void_p(s)), _entry)
+        s = torch.cuda.current_stream(dev).cuda_stream if stream is None else stream.cuda_stream
+        code = getattr(lib(), _entry)(
+            self._h, x_old.data_ptr(), x_unc.data_ptr(), inv_mass.data_ptr(), d.data_ptr(), float(tol), int(max_iter),
+            prec, None if lambda0 is None else lambda0.data_ptr(), x_out.data_ptr(), lambda_out.data_ptr(),
+            iterations_out.data_ptr(), status_out.data_ptr(), s)
+        if code != 0:
+            raise IlvesError(code, _entry)
         return x_out, lambda_out, iterations_out, status_out
 
 
