@@ -252,7 +252,8 @@ struct BatchMol {
     //        d_j -= (L[j,m] inv_m) U[m,j],      -(L[j,m] inv_m) y_m, added to y_j,
     //      and d_j is inverted.  kW lanes take part; in float64 the two lanes of a pair share an
     //      item and take one sum each.  kForward (ILVES-F with its stored factor): y alone.
-    template <int kW, bool kForward, class Sync>
+    //      kOne: no level has more items than kW lanes hold.
+    template <int kW, bool kForward, bool kOne, class Sync>
     __device__ __forceinline__ void eliminate(int l0, int l1, int r, bool& singular, Sync sync) {
         constexpr int kI = kF32 ? kW : kW / 2;
         const int g = kF32 ? r : r >> 1;
@@ -267,11 +268,12 @@ struct BatchMol {
         for (int l = l0; l < l1; ++l) {
             const int hq = lvl_hdr[min(l + 3, l1)];  // levels: this [hb, he), then [he, hn), [hn, hq)
             int k = hb + g;
-            if (k >= he && he + g < hn) {
+            bool mine = k < he;
+            if (!mine && he + g < hn) {
                 h = hdr[he + g];
                 x = terms[HeadWord::first(h)];
             }
-            while (k < he) {
+            while (mine) {
                 const bool diag = HeadWord::diag(h);
                 const int s = (int)HeadWord::slot(h), np = (int)HeadWord::pairs(h);
                 const uint2* tq = terms + HeadWord::first(h) + 1;  // the item's further term pairs
@@ -300,8 +302,9 @@ struct BatchMol {
                 };
                 const uint2 xc = x;
                 k += kI;
-                const int kn = k < he ? k : he + g;
-                const bool more = kn < (k < he ? he : hn);
+                mine = !kOne && k < he;
+                const int kn = mine ? k : he + g;
+                const bool more = kn < (mine ? he : hn);
                 uint32_t h2 = h;
                 if (more) h2 = hdr[kn];
                 x = *tq;  // (unused past the item's last pair; stays in the slice)
@@ -412,14 +415,14 @@ struct BatchMol {
         const int r = tm.rank(), nl = nlevel;
         const auto warp_sync = [] { __syncwarp(); };
         if constexpr (Team::kWarp) {
-            if (nl > 1) eliminate<32, kForward>(1, nl, r, singular, warp_sync);
+            if (nl > 1) eliminate<32, kForward, false>(1, nl, r, singular, warp_sync);
             substitute<32>(0, nl, r, warp_sync);
         } else {
             const auto team_sync = [&] { tm.sync(); };
             const int le = kF32 ? head->wide32 : head->wide16, lb = head->wide_piv;
-            if (le > 1) eliminate<Team::kSize, kForward>(1, le, r, singular, team_sync);
+            if (le > 1) eliminate<Team::kSize, kForward, false>(1, le, r, singular, team_sync);
             if (r < 32) {
-                if (nl > le) eliminate<32, kForward>(le, nl, r, singular, warp_sync);
+                if (nl > le) eliminate<32, kForward, true>(le, nl, r, singular, warp_sync);
                 if (nl > lb) substitute<32>(lb, nl, r, warp_sync);
             }
             if (lb > 0) {

@@ -1404,10 +1404,10 @@ double schedule_cost(const MolHost& M) {
 }
 
 // Time a one-warp team takes per unit of schedule cost (the cost of its 32-lane program),
-// relative to a 96-thread team: calibrated on the 20-200-atom batch (mixed), where 1.2-1.4
-// balanced the two classes' end times and gave the fastest launches (1.8 left the one-warp
-// slots idle for the last ~25 % of the launch).
-constexpr double kNarrowTeamTime = 1.3;
+// relative to a 96-thread team beside it: calibrated on the 20-200-atom batch (mixed; 141 us on
+// 96-thread teams alone), where one-warp teams up to 60 / 70 atoms ran 183 us at 1.3, 154 at
+// 1.7, 145 / 150 at 2.2 and 153 / 156 at 3.0.
+constexpr double kNarrowTeamTime = 2.2;
 
 namespace {
 struct ClassPlan {
