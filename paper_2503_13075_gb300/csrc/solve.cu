@@ -1236,23 +1236,29 @@ __device__ void solve_molecule(const BlockTeam& tm, const MolDesc& D, const uint
 constexpr long long kSpinBudget = 1ll << 22;  // bounded wait: ~0.3 s of polling per launch
 
 // Arrive on a monotone 64-bit counter and wait (bounded) until every CTA of this barrier
-// generation arrived.  Returns false if the wait gave up.
+// generation arrived.  Returns false if the wait gave up.  Thread 0's arrival releases what
+// the CTA wrote (the CTA barrier before it orders the other threads' writes), its last read of
+// the counter acquires what the others wrote; it polls without sleeping at first, since the
+// CTAs arrive within a microsecond or two of each other.
 __device__ __forceinline__ bool grid_sync(unsigned long long* ctr, unsigned n_blocks, long long& budget) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
-        const unsigned long long arrived = atomicAdd(ctr, 1ull) + 1ull;
+        unsigned long long arrived, seen;
+        asm volatile("atom.add.release.gpu.global.u64 %0, [%1], 1;" : "=l"(arrived) : "l"(ctr) : "memory");
+        arrived += 1ull;
         const unsigned long long target = ((arrived + n_blocks - 1) / n_blocks) * (unsigned long long)n_blocks;
         int good = 1;
-        while (*reinterpret_cast<volatile unsigned long long*>(ctr) < target) {
+        for (int polls = 0;; ++polls) {
+            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(ctr) : "memory");
+            if (seen >= target) break;
             if (--budget <= 0) {
                 good = 0;
                 break;
             }
-            __nanosleep(64);
+            if (polls >= 32) __nanosleep(64);
         }
-        __threadfence();
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
         ok = good;
     }
     __syncthreads();
@@ -1648,6 +1654,17 @@ k_solve_parted(const MolDesc* __restrict__ desc, const uint8_t* __restrict__ blo
 // The workspace holds the molecule's positions (SoA; displacements x - x_unc as float-float
 // pairs in the float-float mode), the owned corrections and lambda.
 // ------------------------------------------------------------------------------------
+// The votes of one iteration, read by one thread after a grid barrier and passed on through
+// shared memory (every thread of 450 CTAs reading the same line takes the L2 slice that holds it
+// 3,000 cycles).
+struct Votes { int bad, notconv, singular; };
+__device__ __forceinline__ Votes read_votes(const PartSync* s, int slot) {
+    __shared__ Votes v;
+    if (threadIdx.x == 0) v = Votes{__ldcg(&s->bad[slot]), __ldcg(&s->notconv[slot]), __ldcg(&s->singular[slot])};
+    __syncthreads();
+    return v;
+}
+
 template <class Mode>
 __global__ void __launch_bounds__(kPartThreads, 3)
 k_solve_opm(const MolDesc* __restrict__ desc, const uint8_t* __restrict__ blob, uint8_t* work, PartSync* sync,
@@ -1950,8 +1967,8 @@ k_solve_opm(const MolDesc* __restrict__ desc, const uint8_t* __restrict__ blob, 
             if (CML[p] >> 31) GDL[CML[p] & 0x7FFFFFFFu] = Y[p];
         if (__syncthreads_or(singular) && r0 == 0) atomicOr(&sync->singular[slot], 1);
         if (!(alive = grid_sync(&sync->barrier, nb, budget))) break;
-        const int any_bad = __ldcg(&sync->bad[slot]), any_nc = __ldcg(&sync->notconv[slot]);
-        const int any_sing = __ldcg(&sync->singular[slot]);
+        const Votes votes = read_votes(sync, slot);
+        const int any_bad = votes.bad, any_nc = votes.notconv, any_sing = votes.singular;
         if (dm == 0 && r0 == 0) {  // free the slot used two iterations from now
             sync->notconv[(it + 2) & 3] = 0;
             sync->bad[(it + 2) & 3] = 0;
