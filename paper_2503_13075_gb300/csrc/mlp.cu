@@ -65,7 +65,9 @@ __device__ __forceinline__ float dot3(float3 a, float3 b) { return a.x * b.x + a
 // Prep pass: per-constraint float32 geometry and per-atom weights into the topology's
 // warm-start workspace, so the feature stage gathers 20 bytes per neighbour instead of four
 // float64 atom positions.
+__device__ __forceinline__ void let_next_start();
 __global__ void k_ws_prep(FeatArgs F) {
+    let_next_start();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < F.n_c) {
         const int i = F.con_i[k], j = F.con_j[k];
@@ -157,6 +159,28 @@ __device__ __forceinline__ void copy16(void* smem, const void* gmem) {
                  : "memory");
 }
 __device__ __forceinline__ void copy_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
+// Dependent launches: a kernel launched with launch_after may start while the kernel before it in
+// the stream still runs, once every CTA of that one has passed let_next_start (or ended); what
+// it reads of that kernel's results comes after wait_for_previous, which returns when that
+// kernel has completed.  The set-up of the next kernel (its launch, weights, tensor memory) then
+// overlaps the end of the previous one.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... P, class... A>
+static cudaError_t launch_after(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 
 struct MlpWeights {
     const __nv_bfloat16* w1;  // [NH][NF]  (out x in) bfloat16
@@ -303,6 +327,8 @@ k_mlp_forward(MlpWeights Wt, const float* __restrict__ X, int n, FeatArgs F, flo
     const uint64_t dW1 = smem_desc(saddr_of(sm + SM_W1), 128, (NF / 8) * 128);
     const uint64_t dA2 = smem_desc(saddr_of(sm + SM_A2), 128, (NH / 8) * 128);
     const uint64_t dW2 = smem_desc(saddr_of(sm + SM_W2), 128, (NH / 8) * 128);
+    if constexpr (kFused) wait_for_previous();  // the records of k_ws_prep
+    if constexpr (kTrain) let_next_start();
     uint32_t parity = 0;
     bool ok = true;
     const int n_tiles = (n + TILE - 1) / TILE;
@@ -498,6 +524,8 @@ k_mlp_backward(const float* __restrict__ X, const float* __restrict__ t, int n, 
     float4 gb2 = make_float4(0.f, 0.f, 0.f, 0.f), gw3 = gb2;
     float gb1 = 0.f, gb3 = 0.f, lsum = 0.f;
     const int rb = blockIdx.x * rows_per_cta, re = min(n, rb + rows_per_cta);
+    let_next_start();
+    wait_for_previous();  // the forward's activations
     for (int r0 = rb; r0 < re; r0 += kBwdRows) {
         const int rows = min(kBwdRows, re - r0), rows4 = (rows + 3) & ~3;  // completed with zero rows
         __syncthreads();
@@ -663,6 +691,7 @@ constexpr int kRedThreads = 256;
 __global__ void __launch_bounds__(kRedThreads)
 k_grad_reduce(const float* __restrict__ partial, int n_part, float* __restrict__ grad, float* __restrict__ loss) {
     __shared__ float4 acc[kRedThreads];
+    wait_for_previous();  // the partial gradients
     const int col = blockIdx.x * 32 + (threadIdx.x & 31), row = threadIdx.x >> 5;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     if (col < kPartStride / 4)
@@ -783,6 +812,9 @@ static cudaError_t launch_forward(const MlpWeights& Wt, const float* X, int n, c
     }
     const int tiles = (n + TILE - 1) / TILE;
     const int grid = std::max(1, std::min(tiles, 3 * sms));
+    if constexpr (kFused)  // follows k_ws_prep
+        return launch_after(k_mlp_forward<kFused, kTrain>, grid, kFwdThreads, SM_REQUEST, s, Wt, X, n, F, out, h1, h2, err,
+                            wait_test);
     k_mlp_forward<kFused, kTrain><<<grid, kFwdThreads, SM_REQUEST, s>>>(Wt, X, n, F, out, h1, h2, err, wait_test);
     return cudaGetLastError();
 }
@@ -938,9 +970,10 @@ static ilves_status mlp_gradient(ilves_mlp* M, const float* X, const float* t, i
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
     const int rows = std::max(kBwdMinRows, (n + M->n_part - 1) / M->n_part), parts = (n + rows - 1) / rows;
-    k_mlp_backward<<<parts, kBwdThreads, kBwdSmem, s>>>(X, t, n, rows, M->y, M->h1, M->h2, M->w2b, M->params, M->partial);
-    k_grad_reduce<<<(kPartStride / 4 + 31) / 32, kRedThreads, 0, s>>>(M->partial, parts, grad, loss);
-    return mlp_status(cudaGetLastError());
+    e = launch_after(k_mlp_backward, parts, kBwdThreads, kBwdSmem, s, X, t, n, rows, M->y, M->h1, M->h2, M->w2b, M->params,
+                     M->partial);
+    if (e != cudaSuccess) return mlp_status(e);
+    return mlp_status(launch_after(k_grad_reduce, (kPartStride / 4 + 31) / 32, kRedThreads, 0, s, M->partial, parts, grad, loss));
 }
 
 extern "C" ilves_status ilves_mlp_gradient(ilves_mlp* M, const float* features, const float* target, int32_t n,
