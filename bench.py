@@ -143,7 +143,7 @@ def mixed_fp64_flops(mol_atoms, mol_cons, mol_iters, started):
     return float(np.sum(4 * nc + 10 * nc * (it + 1) + nc * it + (12 * nc + 6 * na) * upd))
 
 
-KERNEL_SOURCES = ("solve.cu", "internal.h", "devmath.cuh", "topology.cpp", "topology_impl.h")
+KERNEL_SOURCES = ("solve.cu", "batched.cuh", "internal.h", "devmath.cuh", "topology.cpp", "topology_impl.h")
 
 
 def kernel_sources_digest():
