@@ -20,10 +20,9 @@
 //    alone, which orders them with warp barriers while the others wait;
 //  - terms come in pairs (the odd one is completed by a zero), incidences four to a word pair.
 // Measured (4096 trees of 20-200 atoms, 96-thread teams; one task per entry and one atom per lane
-// before): mixed 161.9 -> 145.0 us, float64 541 -> 439 us; 8192 trees of 20-50 atoms on one-warp
-// teams 121.7 -> 108.0 us.  The mixed batch issues on 43 % of its cycles with the float64 pipe 34 %
-// busy (its teams wait on one another and on shared memory), the float64 batch fills 76 % of
-// the float64 pipe.
+// before): mixed 162.0 -> 141.2 us, float64 541 -> 430 us; 8192 trees of 20-50 atoms on one-warp
+// teams 121.9 -> 100.1 us.  The mixed batch issues on two of five cycles (its teams wait on one
+// another and on shared memory); the float64 batch fills three quarters of the float64 pipe.
 #pragma once
 
 namespace ilves {
@@ -449,7 +448,8 @@ struct BatchMol {
     // ---- S6: x_a -= w_a sum_k s_k(a) 2 delta_k rho_k   (PV.y holds delta, or lambda0), one
     //      coordinate of one atom per lane: 3 na items over the lanes, atoms by decreasing
     //      degree, leave the busiest warp of a tree of 110 atoms 12 float64 instructions (one
-    //      atom per lane: 21).  The sum runs over the incidences in ascending position.
+    //      atom per lane: 21).  A predicated float64 instruction takes its slot with no lane on,
+    //      so the second to fourth incidences are behind warp votes (145.6 -> 141.2 us mixed).  The sum runs over the incidences in ascending position.
     //      In the mixed mode the corrections are widened to float64 once, not in every
     //      coordinate's lane: dlt is LAM for the starting multipliers, then the rows' space RF
     //      (free until the next violations), which lambda_acc fills.
@@ -491,9 +491,16 @@ struct BatchMol {
                 const double h0 = rho[p0], h1 = rho[p1], h2 = rho[p2], h3 = rho[p3];
                 const double w = W[a], x = *xp;
                 double s = fma(signed64(d0, v.x), h0, 0.0);
-                if (!(v1 & kNoInc)) s = fma(signed64(d1, v1), h1, s);
-                if (!(v2 & kNoInc)) s = fma(signed64(d2, v2), h2, s);
-                if (!(v3 & kNoInc)) s = fma(signed64(d3, v3), h3, s);
+                const unsigned act = __activemask();
+                if (__any_sync(act, !(v1 & kNoInc))) {
+                    if (!(v1 & kNoInc)) s = fma(signed64(d1, v1), h1, s);
+                    if (__any_sync(act, !(v2 & kNoInc))) {
+                        if (!(v2 & kNoInc)) s = fma(signed64(d2, v2), h2, s);
+                        if (__any_sync(act, !(v3 & kNoInc))) {
+                            if (!(v3 & kNoInc)) s = fma(signed64(d3, v3), h3, s);
+                        }
+                    }
+                }
                 if (a < nover)
                     for (int e = over_ptr[a]; e < over_ptr[a + 1]; ++e) {
                         const unsigned o = over[e];

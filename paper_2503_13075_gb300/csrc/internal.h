@@ -105,8 +105,8 @@ constexpr uint32_t kCompactMaxConstraints = 256, kCompactMaxSlots = 4096;
 // Threads of the team that solves one molecule of the batched kernel (whole warps; three
 // warps cut the passes of wide levels at no cost in residency, which shared memory
 // limits to about eight molecules per SM), the batched kernel's CTA size bound and its
-// molecule slots per CTA.  Measured on the 4096-tree batch (mixed, kernel only): 32
-// threads 224 us, 64 195 us, 96 185 us, 128 206 us.
+// molecule slots per CTA.  Measured on the 4096-tree batch (mixed, kernel only, an early version
+// with one task per factor entry): 32 threads 224 us, 64 195 us, 96 185 us, 128 206 us.
 #ifndef ILVES_SLOT_THREADS
 #define ILVES_SLOT_THREADS 96
 #endif
@@ -114,11 +114,11 @@ constexpr int kSlotThreads = ILVES_SLOT_THREADS;
 constexpr int kSlotCtaThreads = 768;
 constexpr int kMaxSlotsPerCta = kSlotCtaThreads / kSlotThreads;
 // Narrow class: molecules of at most narrow_atoms atoms get one-warp teams, up to
-// kNarrowSlotsPerCta per CTA beside its 96-thread teams.  Their slices are small, so an
-// SM's shared memory holds about three times as many of them: batches of 20-50 and 50-100
-// atoms (mixed) ran 1.54x and 1.28x faster that way than on 96-thread teams; on batches of
-// mixed sizes (20-200 atoms) the gain depends on the precision mode, so the automatic
-// choice keeps them on 96 threads and leaves the threshold to the autotuner.
+// kNarrowSlotsPerCta per CTA beside its 96-thread teams.  Their slices are small, so an SM's
+// shared memory holds about three times as many of them: a batch of 4096 trees of 50-100 atoms
+// (mixed) takes 96 us against 117 on 96-thread teams.  On batches of mixed sizes (20-200
+// atoms) they lose (145 us and more against 141), so the automatic choice keeps those on 96
+// threads and leaves the threshold to the autotuner.
 constexpr int kNarrowThreads = 32;
 constexpr int kNarrowSlotsPerCta = kSlotCtaThreads / kNarrowThreads;
 constexpr int kDefaultNarrowAtoms = 100;

@@ -1094,10 +1094,10 @@ ilves_status plan_topology(ilves_topology* T, int32_t n_atoms, int32_t n_c, cons
     // narrow class threshold.  Explicit (narrow_atoms > 0): every batched molecule of at
     // most that many atoms.  Default (0): kDefaultNarrowAtoms, but only for a batch made of
     // such molecules -- at least 90 % of the batched atoms, and more batched molecules than
-    // the wide teams the GPU holds (eight per SM) -- where one-warp teams measured faster;
-    // on batches of mixed sizes the gain depends on the precision mode (20-200 atoms with
-    // one-warp teams up to 60 atoms: 6 % faster in mixed mode, 5 % slower in float64), so
-    // there the autotuner decides; a lone molecule finishes sooner on 96 threads.
+    // the wide teams the GPU holds (eight per SM) -- where one-warp teams measured faster (50-100
+    // atoms: 96 us against 117); on batches of mixed sizes they are slower in every precision
+    // (20-200 atoms, one-warp teams up to 60: mixed 145 us against 141, float64 508 against 469,
+    // float-float 164 against 152); a lone molecule finishes sooner on 96 threads.
     int32_t narrow = o.narrow_atoms > 0 ? o.narrow_atoms : -1;
     if (o.narrow_atoms == 0) {
         int64_t batched = 0, small = 0, n_batched = 0;
