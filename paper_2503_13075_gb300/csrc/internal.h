@@ -405,7 +405,7 @@ ILVES_HD ProgLayout prog_layout(uint32_t na, uint32_t nc, uint32_t ntask, uint32
     return L;
 }
 
-// Numerical state of one molecule (after its program).  Float64-class values (float64,
+// Numerical state of a large molecule, in the workspace.  Float64-class values (float64,
 // or float-float pairs of the same size) take 8 bytes; lp_bytes is the factor element
 // size (4 for float32, 8 for float64); 3-vectors of the factor precision take 4
 // elements and use the fourth: rhof[p].w holds w_i + w_j (the weight of a DIAG entry),
@@ -414,11 +414,8 @@ ILVES_HD ProgLayout prog_layout(uint32_t na, uint32_t nc, uint32_t ntask, uint32
 // With `disp` (float-float mode) the state keeps displacements x - x_unc and the
 // per-constraint differences s_k = x_unc,i - x_unc,j, and rho keeps only the low
 // float parts of rho (the high parts are rhof.xyz).
-// `stage` (= rf, up to the end) is free until the first violation pass: the warp path
-// gathers x_old there (AoS, 24 B per atom) while it sets the molecule up; the region is
-// extended when the arrays after rf are smaller than that.
 struct StateLayout {
-    uint32_t x, w, wl, rho, s, d2, lam, rhof, y, rf, vals, stage, bytes;
+    uint32_t x, w, wl, rho, s, d2, lam, rhof, y, rf, vals, bytes;
 };
 
 ILVES_HD StateLayout state_layout(uint32_t na, uint32_t nc, uint32_t ntask, uint32_t lp_bytes, bool disp) {
@@ -436,9 +433,7 @@ ILVES_HD StateLayout state_layout(uint32_t na, uint32_t nc, uint32_t ntask, uint
     S.y = o;      o = align16(o + (lp_bytes > 4u ? lp_bytes : 4u) * nc);
     S.rf = o;     o = align16(o + vp * nc);
     S.vals = o;   o = align16(o + lp_bytes * ntask);
-    S.stage = S.rf;
-    const uint32_t stage_end = align16(S.stage + 24u * na);
-    S.bytes = o > stage_end ? o : stage_end;
+    S.bytes = o;
     return S;
 }
 

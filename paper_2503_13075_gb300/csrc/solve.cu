@@ -9,9 +9,9 @@
 //   S5  forward substitution fused into the DIAG tasks, backward substitution by level;
 //       lambda += delta
 //   S6  x_a -= w_a sum_{k at a} s_k(a) 2 delta_k rho_k;  back to S2
-// All of a molecule's state lives next to its program: in shared memory for molecules
-// run by one warp (the batched persistent kernel), in a global workspace for large
-// molecules run by a whole CTA.  No host round trip happens inside the Newton loop.
+// All of a molecule's state lives next to its program: in shared memory for the molecules of
+// the batched persistent kernel (batched.cuh), in a global workspace for large molecules run
+// by a whole CTA.  No host round trip happens inside the Newton loop.
 //
 // Precision modes: FP64 runs every step in float64.  MIXED keeps S2, the lambda
 // accumulation and S6 in float64 and runs S3-S5 in float32 (the outer Newton loop is
@@ -26,7 +26,6 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
-#include <type_traits>
 #include <vector>
 
 #include "ilves.h"
