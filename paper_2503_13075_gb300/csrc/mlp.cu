@@ -164,7 +164,9 @@ __device__ __forceinline__ void copy_wait_all() { asm volatile("cp.async.wait_al
 // the stream still runs, once every CTA of that one has passed let_next_start (or ended); what
 // it reads of that kernel's results comes after wait_for_previous, which returns when that
 // kernel has completed.  The set-up of the next kernel (its launch, weights, tensor memory) then
-// overlaps the end of the previous one.
+// overlaps the end of the previous one.  A dependent kernel is resident while those results are
+// written, so they are not constant for its life: it takes them by plain pointers (no const
+// __restrict__, no __ldg), whose loads stay behind the wait and go through the coherent path.
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <class... P, class... A>
@@ -490,9 +492,9 @@ __device__ __forceinline__ float2 fma2(float a, float2 b, float2 c) {
     return d;
 }
 __global__ void __launch_bounds__(kBwdThreads, 1)
-k_mlp_backward(const float* __restrict__ X, const float* __restrict__ t, int n, int rows_per_cta,
-               const float* __restrict__ y, const __nv_bfloat16* __restrict__ h1, const float* __restrict__ h2,
-               const __nv_bfloat16* __restrict__ w2b, const float* __restrict__ params, float* __restrict__ partial) {
+k_mlp_backward(const float* __restrict__ X, const float* __restrict__ t, int n, int rows_per_cta, const float* y,
+               const __nv_bfloat16* h1, const float* h2, const __nv_bfloat16* __restrict__ w2b,
+               const float* __restrict__ params, float* __restrict__ partial) {
     extern __shared__ __align__(16) float bsm[];
     float* w2s = bsm;                       // [c][k], the bfloat16 weights the forward used
     float* dzs = w2s + NH * NH;             // dz2 [r][c], then dz1 [r][k]
@@ -545,7 +547,7 @@ k_mlp_backward(const float* __restrict__ X, const float* __restrict__ t, int n, 
                                                    : make_float4(0.f, 0.f, 0.f, 0.f);
         for (int e = tid; e < rows4 * (NH / 8); e += kBwdThreads) {
             uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (e < rows * (NH / 8)) v = __ldg(reinterpret_cast<const uint4*>(h1 + (int64_t)r0 * NH) + e);
+            if (e < rows * (NH / 8)) v = reinterpret_cast<const uint4*>(h1 + (int64_t)r0 * NH)[e];
             const __nv_bfloat162* b = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
             for (int q = 0; q < 4; ++q) *reinterpret_cast<float2*>(h1s + 8 * e + 2 * q) = __bfloat1622float2(b[q]);
@@ -557,7 +559,7 @@ k_mlp_backward(const float* __restrict__ X, const float* __restrict__ t, int n, 
             for (int q = 0; q < kBwdRows / 8; ++q) {
                 const int r = r8 + 8 * q;
                 h[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (r < rows) h[q] = __ldg(reinterpret_cast<const float4*>(h2 + (int64_t)(r0 + r) * NH + c4));
+                if (r < rows) h[q] = *reinterpret_cast<const float4*>(h2 + (int64_t)(r0 + r) * NH + c4);
             }
 #pragma unroll
             for (int q = 0; q < kBwdRows / 8; ++q) {
@@ -598,7 +600,7 @@ k_mlp_backward(const float* __restrict__ X, const float* __restrict__ t, int n, 
         for (int a = 0; a < 4; ++a)
 #pragma unroll
             for (int b = 0; b < 4; ++b) dh[a][b] = make_float2(0.f, 0.f);
-        if (ty < rows4) {  // rows past rows4 hold an earlier chunk's values: computed, not stored
+        if (ty < rows4) {  // rows past rows4 repeat the last one: computed, not stored
 #pragma unroll 1
             for (int cc = 0; cc < NH; cc += 4) {
                 float av[4][4];
@@ -689,7 +691,7 @@ k_mlp_backward(const float* __restrict__ X, const float* __restrict__ t, int n, 
 // each add every eighth partial, then one adds the eight.
 constexpr int kRedThreads = 256;
 __global__ void __launch_bounds__(kRedThreads)
-k_grad_reduce(const float* __restrict__ partial, int n_part, float* __restrict__ grad, float* __restrict__ loss) {
+k_grad_reduce(const float* partial, int n_part, float* __restrict__ grad, float* __restrict__ loss) {
     __shared__ float4 acc[kRedThreads];
     wait_for_previous();  // the partial gradients
     const int col = blockIdx.x * 32 + (threadIdx.x & 31), row = threadIdx.x >> 5;
@@ -697,7 +699,7 @@ k_grad_reduce(const float* __restrict__ partial, int n_part, float* __restrict__
     if (col < kPartStride / 4)
 #pragma unroll 8
         for (int p = row; p < n_part; p += kRedThreads / 32) {
-            const float4 v = __ldg(reinterpret_cast<const float4*>(partial + (int64_t)p * kPartStride) + col);
+            const float4 v = reinterpret_cast<const float4*>(partial + (int64_t)p * kPartStride)[col];
             s.x += v.x;
             s.y += v.y;
             s.z += v.z;
