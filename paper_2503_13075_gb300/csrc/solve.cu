@@ -2259,8 +2259,8 @@ static ilves_status upload_topology(ilves_topology* T, const ilves_setup_opts& o
     // per slot) comes off the per-block limit
     const int arena = std::min(smem_optin - kStaticSlotSmem, smem_sm / ctas_per_sm - 1024) & ~15;
     // molecules whose slice does not fit an arena take the CTA-per-molecule path
-    for (auto& M : T->mols)
-        if (!M.large && footprint(M, ILVES_PREC_FP64) > (uint32_t)arena) M.large = true;
+    for (int32_t m = 0; m < T->n_mol; ++m)
+        if (!T->mols[m].large && footprint(T->mols[m], ILVES_PREC_FP64) > (uint32_t)arena) leave_batched(T, m);
     // descriptors, program blobs, atom ids
     std::vector<int32_t> order;
     for (int32_t m = 0; m < T->n_mol; ++m)

@@ -1001,6 +1001,26 @@ static void relabel_atoms_by_degree(MolHost& M, Program& P) {
     }
 }
 
+// A batched molecule whose slice does not fit an arena takes the CTA-per-molecule path.  The
+// kernels of that path take local atom a as the molecule's a-th atom in ascending global order,
+// so the labels by degree are undone, in the constraints and in the program's shared atoms.
+void leave_batched(ilves_topology* T, int32_t m) {
+    MolHost& M = T->mols[m];
+    for (size_t c = 0; c < M.ci.size(); ++c) {
+        M.ci[c] = M.aperm[M.ci[c]];
+        M.cj[c] = M.aperm[M.cj[c]];
+    }
+    for (TaskW& w : T->progs[m]->tasks) {
+        const uint32_t a = w.atomsign >> 1;
+        if (w.atomsign != kNoAtom32 && a < (uint32_t)M.aperm.size())
+            w.atomsign = ((uint32_t)M.aperm[a] << 1) | (w.atomsign & 1u);
+    }
+    M.aperm.clear();
+    M.bsz = BatchSizes{};
+    M.team = kSlotThreads;
+    M.large = true;
+}
+
 // true if a program fits the batched kernel's encoding: value slots, terms per item (pivots and
 // entries of U; those of L share their terms) and term pairs fit their fields
 static bool fits_compact(const Program& P) {

@@ -128,6 +128,7 @@ namespace ilves {
 ilves_status plan_topology(ilves_topology* T, int32_t n_atoms, int32_t n_c, const int32_t* ai,
                            const int32_t* aj, const ilves_setup_opts& o);
 uint32_t footprint(const MolHost& M, int mode);
+void leave_batched(ilves_topology* T, int32_t m);
 double schedule_cost(const MolHost& M);
 void build_batched_schedule(ilves_topology* T, int mode, int32_t n_cta, int32_t warps, int32_t arena,
                             HostSchedule& S);
