@@ -449,17 +449,43 @@ struct BatchMol {
     //      coordinate of one atom per lane: 3 na items over the lanes, atoms by decreasing
     //      degree, leave the busiest warp of a tree of 110 atoms 12 float64 instructions (one
     //      atom per lane: 21).  A predicated float64 instruction takes its slot with no lane on,
-    //      so the second to fourth incidences are behind warp votes (145.6 -> 141.2 us mixed).  The sum runs over the incidences in ascending position.
+    //      so the second to fourth incidences are behind warp votes (145.6 -> 141.2 us mixed).
+    //      The sum runs over the incidences in ascending position.
     //      In the mixed mode the corrections are widened to float64 once, not in every
     //      coordinate's lane: dlt is LAM for the starting multipliers, then the rows' space RF
     //      (free until the next violations), which lambda_acc fills.
     __device__ __forceinline__ static double signed64(double v, unsigned inc) {
         return __hiloint2double(__double2hiint(v) ^ (int)(inc << 31), __double2loint(v));
     }
-    __device__ __forceinline__ void term_df(unsigned v, int c, dfloat& s) const {
+    // The float-float mode takes a whole atom per lane: its terms are float32 instructions, of which
+    // no warp has too few lanes on, and three lanes to an atom would repeat the incidence, the
+    // correction and the loop (4096 / 1001 trees, diagonal start: 150.8 / 52.3 us by coordinates,
+    // 148.8 / 50.1 by atoms).
+    struct Sum3 { dfloat x, y, z; };
+    __device__ __forceinline__ void term_df(unsigned v, Sum3& s) const {
         const int p = (int)((v >> 1) & 0xFFu);
         const float dl = (float)PV[p].y, k = (v & 1u) ? -(dl + dl) : (dl + dl);
-        s = df_add(s, df_mul_f(dfloat{reinterpret_cast<const float*>(RHOF + p)[c], RHOL[c * nc + p]}, k));
+        const V4 hi = RHOF[p];
+        s.x = df_add(s.x, df_mul_f(dfloat{(float)hi.x, RHOL[p]}, k));
+        s.y = df_add(s.y, df_mul_f(dfloat{(float)hi.y, RHOL[nc + p]}, k));
+        s.z = df_add(s.z, df_mul_f(dfloat{(float)hi.z, RHOL[2 * nc + p]}, k));
+    }
+    __device__ __forceinline__ void update_df(int r0, int ts) {
+        for (int a = r0; a < na; a += ts) {
+            const uint2 v = inc4[a];
+            const unsigned v1 = v.x >> 16, v2 = v.y & 0xFFFFu, v3 = v.y >> 16;
+            Sum3 s{{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+            term_df(v.x, s);
+            if (!(v1 & kNoInc)) term_df(v1, s);
+            if (!(v2 & kNoInc)) term_df(v2, s);
+            if (!(v3 & kNoInc)) term_df(v3, s);
+            if (a < nover)
+                for (int e = over_ptr[a]; e < over_ptr[a + 1]; ++e) term_df(over[e], s);
+            const dfloat w = as_df(W[a]);
+            X[a] = as_bits(df_sub(as_df(X[a]), df_mul(w, s.x)));
+            X[na + a] = as_bits(df_sub(as_df(X[na + a]), df_mul(w, s.y)));
+            X[2 * na + a] = as_bits(df_sub(as_df(X[2 * na + a]), df_mul(w, s.z)));
+        }
     }
     template <int kStride>
     __device__ __forceinline__ void update(const double* dlt, int r0, int ts) {
@@ -472,43 +498,32 @@ struct BatchMol {
             if (q + ts < n) rec = inc4[(q + ts) / 3];
             double* xp = X + c * na + a;
             const unsigned v1 = v.x >> 16, v2 = v.y & 0xFFFFu, v3 = v.y >> 16;
-            if constexpr (DF) {
-                dfloat s{0.f, 0.f};
-                term_df(v.x, c, s);
-                if (!(v1 & kNoInc)) term_df(v1, c, s);
-                if (!(v2 & kNoInc)) term_df(v2, c, s);
-                if (!(v3 & kNoInc)) term_df(v3, c, s);
-                if (a < nover)
-                    for (int e = over_ptr[a]; e < over_ptr[a + 1]; ++e) term_df(over[e], c, s);
-                *xp = as_bits(df_sub(as_df(*xp), df_mul(as_df(W[a]), s)));
-            } else {
-                // the four products' operands first, then the float64 chain
-                const int p0 = (int)((v.x >> 1) & 0xFFu), p1 = (int)((v1 >> 1) & 0xFFu);
-                const int p2 = (int)((v2 >> 1) & 0xFFu), p3 = (int)((v3 >> 1) & 0xFFu);
-                const double* rho = RHO + c * nc;
-                const double d0 = dlt[kStride * p0], d1 = dlt[kStride * p1], d2 = dlt[kStride * p2],
-                             d3 = dlt[kStride * p3];
-                const double h0 = rho[p0], h1 = rho[p1], h2 = rho[p2], h3 = rho[p3];
-                const double w = W[a], x = *xp;
-                double s = fma(signed64(d0, v.x), h0, 0.0);
-                const unsigned act = __activemask();
-                if (__any_sync(act, !(v1 & kNoInc))) {
-                    if (!(v1 & kNoInc)) s = fma(signed64(d1, v1), h1, s);
-                    if (__any_sync(act, !(v2 & kNoInc))) {
-                        if (!(v2 & kNoInc)) s = fma(signed64(d2, v2), h2, s);
-                        if (__any_sync(act, !(v3 & kNoInc))) {
-                            if (!(v3 & kNoInc)) s = fma(signed64(d3, v3), h3, s);
-                        }
+            // the four products' operands first, then the float64 chain
+            const int p0 = (int)((v.x >> 1) & 0xFFu), p1 = (int)((v1 >> 1) & 0xFFu);
+            const int p2 = (int)((v2 >> 1) & 0xFFu), p3 = (int)((v3 >> 1) & 0xFFu);
+            const double* rho = RHO + c * nc;
+            const double d0 = dlt[kStride * p0], d1 = dlt[kStride * p1], d2 = dlt[kStride * p2],
+                         d3 = dlt[kStride * p3];
+            const double h0 = rho[p0], h1 = rho[p1], h2 = rho[p2], h3 = rho[p3];
+            const double w = W[a], x = *xp;
+            double s = fma(signed64(d0, v.x), h0, 0.0);
+            const unsigned act = __activemask();
+            if (__any_sync(act, !(v1 & kNoInc))) {
+                if (!(v1 & kNoInc)) s = fma(signed64(d1, v1), h1, s);
+                if (__any_sync(act, !(v2 & kNoInc))) {
+                    if (!(v2 & kNoInc)) s = fma(signed64(d2, v2), h2, s);
+                    if (__any_sync(act, !(v3 & kNoInc))) {
+                        if (!(v3 & kNoInc)) s = fma(signed64(d3, v3), h3, s);
                     }
                 }
-                if (a < nover)
-                    for (int e = over_ptr[a]; e < over_ptr[a + 1]; ++e) {
-                        const unsigned o = over[e];
-                        const int p = (int)((o >> 1) & 0xFFu);
-                        s = fma(signed64(dlt[kStride * p], o), rho[p], s);
-                    }
-                *xp = fma(-w, s, x);
             }
+            if (a < nover)
+                for (int e = over_ptr[a]; e < over_ptr[a + 1]; ++e) {
+                    const unsigned o = over[e];
+                    const int p = (int)((o >> 1) & 0xFFu);
+                    s = fma(signed64(dlt[kStride * p], o), rho[p], s);
+                }
+            *xp = fma(-w, s, x);
         }
     }
     __device__ __forceinline__ void lambda_acc(int p) {
@@ -557,7 +572,8 @@ __device__ void solve_batched(const Team& tm, const MolDesc& D, const BatchLayou
         tm.sync();
     }
     if (A.has_start()) {  // x = x_unc - M^-1 G(x_old)^T lambda0
-        if constexpr (Mode::df || sizeof(typename Mode::LP) == 8) M.template update<2>(M.corrections(), r0, ts);
+        if constexpr (Mode::df) M.update_df(r0, ts);
+        else if constexpr (sizeof(typename Mode::LP) == 8) M.template update<2>(M.corrections(), r0, ts);
         else M.template update<1>(M.LAM, r0, ts);
         tm.sync();
     }
@@ -593,7 +609,8 @@ __device__ void solve_batched(const Team& tm, const MolDesc& D, const BatchLayou
         if constexpr (Team::kWarp) tm.sync();
         for (int p = r0; p < nc; p += ts) M.lambda_acc(p);
         if constexpr (!Mode::df && sizeof(typename Mode::LP) == 4) tm.sync();
-        M.template update<2>(M.corrections(), r0, ts);
+        if constexpr (Mode::df) M.update_df(r0, ts);
+        else M.template update<2>(M.corrections(), r0, ts);
         tm.sync();
     }
     M.out_atoms(r0, ts);
