@@ -18,7 +18,12 @@
 //    the current one;
 //  - levels of at most 32 items or pivots, the last ones, belong to the team's first warp
 //    alone, which orders them with warp barriers while the others wait;
-//  - terms come in pairs (the odd one is completed by a zero), incidences four to a word pair.
+//  - terms come in pairs (the odd one is completed by a zero), incidences four to a word pair;
+//  - no pass is unrolled.  Eight teams are in different passes at any time, and both classes of
+//    teams and both kinds of solve have code of their own, so the passes' code has to stay in the
+//    instruction caches: unrolled four times by the compiler, 1.5 (float-float) and 0.6 (mixed)
+//    of a warp's stall cycles an issue were waits for instructions, 1.7 and 0.9 with one-warp teams
+//    beside the others; now 0.7 and 0.3 (135 -> 127 us mixed, 151 -> 129 us float-float).
 // Measured (4096 trees of 20-200 atoms, 96-thread teams; one task per entry and one atom per lane
 // before): mixed 162.0 -> 141.2 us, float64 541 -> 430 us; 8192 trees of 20-50 atoms on one-warp
 // teams 121.9 -> 100.1 us.  The mixed batch issues on two of five cycles (its teams wait on one
@@ -34,6 +39,9 @@ struct BatchMol {
     struct alignas(2 * sizeof(LP)) V2 { LP x, y; };
     static constexpr bool DF = Mode::df;
     static constexpr bool kF32 = sizeof(LP) == 4;
+    // loops of copies: two at a time, except in the float-float mode, whose code is the largest
+    // (4096 chains of 64 atoms, mixed: 81.3 -> 79.8 us; 4096 trees, float-float: 128.9 against 131.8)
+    static constexpr int kCopies = DF ? 1 : 2;
     int na, nc, npair, nlevel, nover, zero;
     const BatchHead* head;
     const uint32_t* con;  // local atoms i | j << 16 of each position
@@ -108,17 +116,20 @@ struct BatchMol {
     //      start); inv_mass -> W, d -> D2, lambda0 -> LAM as raw values.  The reads run over atom
     //      slots, so consecutive lanes read consecutive addresses.
     __device__ __forceinline__ void s1_gather(int r0, int ts) {
+#pragma unroll 1
         for (int p = r0; p < nc; p += ts) {
             const int32_t g = gid_of_con(p);
             cp_async8(D2 + p, A.d + g);
             if (A.lambda0 && !A.start_diag) cp_async4(LAM + p, A.lambda0 + g);
         }
+#pragma unroll kCopies
         for (int e = r0; e < 3 * na; e += ts) {
             const int o = e / 3, c = e - 3 * o, a = (int)aslot[o];
             const int64_t g = 3 * slot_gid(o) + c;
             cp_async8(STG + 3 * a + c, A.x_old + g);
             cp_async8(DF ? X + 3 * a + c : X + c * na + a, A.x_unc + g);
         }
+#pragma unroll kCopies
         for (int o = r0; o < na; o += ts) cp_async8(W + aslot[o], A.inv_mass + slot_gid(o));
         cp_async_wait_all();
     }
@@ -231,6 +242,7 @@ struct BatchMol {
     __device__ __forceinline__ void assemble(const V4* R, int r0, int ts, bool& singular) {
         if (r0 == 0) C[zero] = V2{LP(0), LP(0)};
         const int n0 = lvl_piv[1];
+#pragma unroll 1
         for (int p = r0; p < nc; p += ts) {
             const V4 rr = R[p], pp = RHOF[p];
             LP a = pp.w * dot(rr, pp);
@@ -240,6 +252,7 @@ struct BatchMol {
             }
             PV[p].x = a;
         }
+#pragma unroll 1
         for (int k = r0; k < npair; k += ts) {
             const uint32_t w = pairs[k];
             const int j = (int)PairWord::row(w), q = (int)PairWord::col(w);
@@ -276,6 +289,7 @@ struct BatchMol {
             const int hq = lvl_hdr[min(l + 3, l1)];  // levels: this [hb, he), then [he, hn), [hn, hq)
             if constexpr (!kF32 && !kForward) {
                 const int s1 = (int)BackWord::slot(back[lvl_piv[l]]);
+#pragma unroll 1
                 for (int k = (int)BackWord::slot(back[lvl_piv[l - 1]]) + r; k < s1; k += kW)
                     C[k].y *= PV[PairWord::row(pairs[k])].x;
                 sync();
@@ -324,6 +338,7 @@ struct BatchMol {
                 if (!kForward || diag) {
                     term(xc.x);
                     term(xc.y);
+#pragma unroll 1
                     for (int q = 1; q < np; ++q) {
                         const uint2 xn = x;
                         x = *++tq;
@@ -388,6 +403,7 @@ struct BatchMol {
             if (k < nu) d -= o.u[k] * z[k];
         if (nu > 4) {
             const int us = (int)BackWord::slot(o.rec);
+#pragma unroll 1
             for (int k = 4; k < nu; ++k) d -= C[us + k].x * PV[PairWord::col(pairs[us + k])].y;
         }
         PV[p].y = d * o.v.x;
@@ -407,6 +423,7 @@ struct BatchMol {
             if (next) nxt.rec = back[pn + r];
             if (pb + r < pe) finish_pivot(cur, pb + r);
             if (next) fetch_values(nxt, pn + r);
+#pragma unroll 1
             for (int p = pb + r + kW; p < pe; p += kW) {
                 Ahead o;
                 o.rec = back[p];
@@ -471,6 +488,7 @@ struct BatchMol {
         s.z = df_add(s.z, df_mul_f(dfloat{(float)hi.z, RHOL[2 * nc + p]}, k));
     }
     __device__ __forceinline__ void update_df(int r0, int ts) {
+#pragma unroll 1
         for (int a = r0; a < na; a += ts) {
             const uint2 v = inc4[a];
             const unsigned v1 = v.x >> 16, v2 = v.y & 0xFFFFu, v3 = v.y >> 16;
@@ -480,6 +498,7 @@ struct BatchMol {
             if (!(v2 & kNoInc)) term_df(v2, s);
             if (!(v3 & kNoInc)) term_df(v3, s);
             if (a < nover)
+#pragma unroll 1
                 for (int e = over_ptr[a]; e < over_ptr[a + 1]; ++e) term_df(over[e], s);
             const dfloat w = as_df(W[a]);
             X[a] = as_bits(df_sub(as_df(X[a]), df_mul(w, s.x)));
@@ -492,6 +511,7 @@ struct BatchMol {
         const int n = 3 * na;
         uint2 rec = make_uint2(0u, 0u);
         if (r0 < n) rec = inc4[r0 / 3];
+#pragma unroll 1
         for (int q = r0; q < n; q += ts) {
             const int a = q / 3, c = q - 3 * a;
             const uint2 v = rec;
@@ -518,6 +538,7 @@ struct BatchMol {
                 }
             }
             if (a < nover)
+#pragma unroll 1
                 for (int e = over_ptr[a]; e < over_ptr[a + 1]; ++e) {
                     const unsigned o = over[e];
                     const int p = (int)((o >> 1) & 0xFFu);
@@ -541,6 +562,7 @@ struct BatchMol {
 
     // ---- S7: the positions, one coordinate per lane in global order; the multipliers
     __device__ __forceinline__ void out_atoms(int r0, int ts) {
+#pragma unroll kCopies
         for (int e = r0; e < 3 * na; e += ts) {
             const int o = e / 3, c = e - 3 * o, a = (int)aslot[o];
             const int64_t g = 3 * slot_gid(o) + c;
@@ -562,12 +584,15 @@ __device__ void solve_batched(const Team& tm, const MolDesc& D, const BatchLayou
     // ---- S1
     M.s1_gather(r0, ts);
     tm.sync();
+#pragma unroll 1
     for (int a = r0; a < na; a += ts) M.s1_atom(a);
     if (r0 == 0) M.s1_dummy();
     tm.sync();
+#pragma unroll 1
     for (int p = r0; p < nc; p += ts) M.s1_constraint(p);
     tm.sync();
     if constexpr (Mode::df) {  // displacements start at zero
+#pragma unroll 1
         for (int q = r0; q < 3 * na; q += ts) M.X[q] = 0.0;
         tm.sync();
     }
@@ -580,6 +605,7 @@ __device__ void solve_batched(const Team& tm, const MolDesc& D, const BatchLayou
     int status = ILVES_MOL_MAX_ITER, iters = A.max_iter;
     for (int it = 0;; ++it) {
         bool conv = true, bad = false;
+#pragma unroll 1
         for (int p = r0; p < nc; p += ts) M.violation(p, M.con[p], conv, bad, !A.chord);
         if (tm.all(conv && !bad)) {
             status = ILVES_MOL_CONVERGED;
@@ -607,6 +633,7 @@ __device__ void solve_batched(const Team& tm, const MolDesc& D, const BatchLayou
             break;
         }
         if constexpr (Team::kWarp) tm.sync();
+#pragma unroll 1
         for (int p = r0; p < nc; p += ts) M.lambda_acc(p);
         if constexpr (!Mode::df && sizeof(typename Mode::LP) == 4) tm.sync();
         if constexpr (Mode::df) M.update_df(r0, ts);
@@ -615,6 +642,7 @@ __device__ void solve_batched(const Team& tm, const MolDesc& D, const BatchLayou
     }
     M.out_atoms(r0, ts);
     if (A.lambda_out)
+#pragma unroll 1
         for (int p = r0; p < nc; p += ts) M.out_lambda(p);
     if (r0 == 0) {
         if (A.iterations_out) A.iterations_out[D.mol_id] = iters;
