@@ -1424,10 +1424,17 @@ double schedule_cost(const MolHost& M) {
 }
 
 // Time a one-warp team takes per unit of schedule cost (the cost of its 32-lane program),
-// relative to a 96-thread team beside it: calibrated on the 20-200-atom batch (mixed; 141 us on
-// 96-thread teams alone), where one-warp teams up to 60 / 70 atoms ran 183 us at 1.3, 154 at
-// 1.7, 145 / 150 at 2.2 and 153 / 156 at 3.0.
-constexpr double kNarrowTeamTime = 2.2;
+// relative to a 96-thread team beside it.  Small molecules want more (batches of one size: 1.8 for
+// 40 atoms), large ones less (1.0 for 100, 0.85 for 160: their cost counts a pass for every 32
+// tasks, and one warp keeps its pace through them).  Measured on 4096 trees of 20-200 atoms, one-warp
+// teams up to 40 / 60 / 80 / 100 / 130 / 160 atoms (us):
+//            mixed                              float64                            float-float
+//   1.1   141 / 129 / 127 / 130 / 144 / 153   410 / 436 / 422 / 425 / 432 / 505   151 / 157 / 151 / 153 / 158 / 167
+//   1.6   131 / 126 / 129 / 150 / 152 / 153   409 / 435 / 457 / 493 / 516 / 608   133 / 143 / 151 / 157 / 159 / 165
+//   2.2   131 / 133 / 142 / 153 / 187 / 234   408 / 435 / 457 / 492 / 516 / 608   132 / 138 / 148 / 156 / 200 / 238
+// (96-thread teams alone: 127, 413, 129).  With 2.2 the planner took almost every 96-thread slot
+// from the large molecules once the threshold passed 100 atoms.
+constexpr double kNarrowTeamTime = 1.6;
 
 namespace {
 struct ClassPlan {
