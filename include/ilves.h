@@ -119,9 +119,12 @@ typedef struct {
                                 -2 = plan on the host only: no CUDA call, ilves_solve refused) */
     int32_t max_warp_constraints; /* molecules larger than this use the multi-warp path (0 = auto) */
     int32_t partition_min_constraints; /* molecules with at least this many constraints are
-                                          partitioned over many CTAs (0 = automatic: 4096, or 1000
-                                          for a topology's only molecule past the batched kernel's
-                                          limits; overlapping domains from 4096 on) */
+                                          partitioned over many CTAs (0 = automatic: 4096, and from
+                                          1000 on a topology's only molecule past the batched kernel's
+                                          limits if its parts leave few enough separators to be
+                                          faster than one CTA, and fit the static scratch array of
+                                          ilves_solve_static_scratch; overlapping domains from 4096
+                                          on) */
     int32_t part_constraints;      /* target constraints per part of a partitioned molecule (0 = 256) */
     int32_t wait_test;             /* testing only (0 in normal use): the grid barriers of partitioned
                                       solves also wait for this many CTAs that do not exist, so every

@@ -437,6 +437,8 @@ ILVES_HD StateLayout state_layout(uint32_t na, uint32_t nc, uint32_t ntask, uint
     return S;
 }
 
+constexpr size_t kStaticScratchBytes = size_t(16) << 20;  // see ilves_solve_static_scratch
+
 // One molecule as the kernels see it.
 struct MolDesc {
     int64_t blob_off;    // byte offset of the program blob in the blob buffer (16-B aligned)

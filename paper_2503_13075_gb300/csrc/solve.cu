@@ -2558,7 +2558,6 @@ static ilves_status launch_mode(ilves_topology* T, const SolveArgs& A, cudaStrea
 // host-side stand-in); its device address is looked up on every call, so a device reset
 // between calls cannot leave a stale address behind.
 // ------------------------------------------------------------------------------------
-constexpr size_t kStaticScratchBytes = size_t(16) << 20;
 static __device__ __align__(256) uint8_t g_static_scratch[kStaticScratchBytes];
 
 // Device address of g_static_scratch on the current device.

@@ -21,6 +21,7 @@
 #include <cstdint>
 #include <cstring>
 #include <iterator>
+#include <memory>
 #include <numeric>
 #include <queue>
 #include <vector>
@@ -1035,6 +1036,102 @@ static bool fits_compact(const Program& P) {
 }
 
 // ------------------------------------------------------------------------------------
+// partitioned molecules
+// ------------------------------------------------------------------------------------
+// The program of a partitioned molecule; nullptr if the cuts leave more than max_sep separators.
+static Program* compile_parted(int32_t na, int32_t nc, const std::vector<std::vector<int32_t>>& adj,
+                               const std::vector<int32_t>& ci, const std::vector<int32_t>& cj,
+                               const ilves_setup_opts& o, int32_t n_sm, int32_t max_sep) {
+    // automatic part size: about 256 constraints, but never more parts (plus the
+    // separator CTA) than three CTAs per SM can keep resident, since the parts of a
+    // cooperative launch run at once with their programs in shared memory
+    int32_t part_size = o.part_constraints > 0 ? o.part_constraints : 256;
+    if (o.part_constraints <= 0) {
+        const int32_t max_parts = 3 * n_sm - 1;
+        part_size = std::max(part_size, (nc + max_parts - 1) / max_parts);
+    }
+    const int32_t n_parts = std::max(2, std::min(8192, (nc + part_size - 1) / part_size));
+    std::vector<int32_t> bounds = partition_atoms(na, ci, cj, n_parts);
+    const int32_t np = (int32_t)bounds.size() - 1;
+    std::vector<int32_t> part_of(na);
+    for (int32_t q = 0; q < np; ++q)
+        for (int32_t a = bounds[q]; a < bounds[q + 1]; ++a) part_of[a] = q;
+    std::vector<int32_t> seg(nc);
+    std::vector<int8_t> stage(nc);
+    int32_t n_sep = 0;
+    for (int32_t c = 0; c < nc; ++c) {
+        const bool inner = part_of[ci[c]] == part_of[cj[c]];
+        seg[c] = inner ? part_of[ci[c]] : np;
+        stage[c] = inner ? 0 : 1;
+        n_sep += stage[c];
+    }
+    if (n_sep > max_sep) return nullptr;
+    std::vector<int32_t> seg_atom(bounds);
+    seg_atom.push_back(na);  // the separator segment owns no atoms
+    // elimination order: rounds of independent pivots of near-minimum degree; the
+    // degree slack is tuned per molecule for the fewest levels in the deepest part
+    // (every level of a part costs a CTA barrier and a dependent chain, twice per
+    // iteration), then the fewest terms
+    Program* P = nullptr;
+    int64_t best_key = 0;
+    for (int32_t slack : {2, 3, 4, 6}) {
+        Program C = compile(nc, eliminate_rounds(nc, adj, slack, false, &stage), ci, cj, 256, na, &seg, np + 1, &seg_atom);
+        int32_t deepest = 0;
+        for (int32_t q = 0; q < np; ++q) deepest = std::max(deepest, C.seg_lvl[q + 1] - 1 - C.seg_lvl[q]);
+        const int64_t key = ((int64_t)deepest << 40) + (int64_t)C.terms.size();
+        if (!P || key < best_key) {
+            delete P;
+            P = new Program(std::move(C));
+            best_key = key;
+        }
+    }
+    return P;
+}
+
+// Partition a topology's only molecule of [kLonePartitionMin, 4096) constraints, past the batched
+// kernel's limits, that one CTA could solve?  Its parts run on several SMs, where one CTA has one
+// SM's float64 pipe, but they cost four grid barriers an iteration and the separators are
+// eliminated level by level on one CTA.  (Several such molecules share one launch of a CTA each,
+// while partitioned solves run one after another.)  Measured (us, mixed / float64 / float-float,
+// zero start; one CTA against parts):
+//  - molecules without dense blocks: about 5 us a separator level.  Trees of 1002 atoms with 7, 10
+//    and 11 levels: 161 / 261 / 146 against 150 / 247 / 152, 172 / 276 / 154 against 165 / 274 / 167,
+//    159 / 256 / 144 against 177 / 301 / 178; of 1100 atoms with 11 and 14: 185 / 305 / 171 against
+//    161 / 265 / 162, 186 / 301 / 164 against 175 / 312 / 175; of 1300 with 14: 192 / 309 / 179
+//    against 174 / 302 / 173; of 4000 with 24: 495 / 770 / 451 against 224 / 404 / 226.  Chains and
+//    protein-like molecules have 2 to 4 (1010 atoms: 146 / 219 / 137 against 116 / 173 / 115).  The
+//    two sides meet at 8 levels for 1000 constraints and 3 more for each further 100.
+//  - above that line the elimination's terms decide, those of the largest part and of the
+//    separators against all of one CTA's: a third of the time at a seventeenth (strip of
+//    100 x 4 x 4 atoms, 142 levels: 142 ms against 16 ms), no gain at 0.44 (24 x 24 atoms, 73
+//    levels: 5.1 / 8.4 / 5.1 ms against 5.0 / 6.6 / 5.3).
+//  - grids whose cuts leave hundreds of separators are slower in parts, and much slower to plan
+//    (8 x 8 x 8 atoms, 352 separators: 48 against 60 ms; 4 x 4 x 40, 683: 24 against 315 ms; 2 x 2 x
+//    300, 849 levels: planned in 0.2 against 30 s): past kLoneMaxSeparators no partition is planned.
+constexpr int32_t kLonePartitionMin = 1000, kLoneMaxSeparators = 256;
+static bool lone_partition_pays(const Program& P, int32_t na, int32_t nc, const std::vector<std::vector<int32_t>>& adj,
+                                const std::vector<int32_t>& ci, const std::vector<int32_t>& cj,
+                                const ilves_setup_opts& o, std::unique_ptr<Program>& one_cta) {
+    const int32_t np = P.n_seg - 1;
+    // nothing that the static scratch array held may stop fitting it
+    const int64_t state = std::max(state_layout(na, nc, (uint32_t)P.tasks.size(), 8, false).bytes,
+                                   state_layout(na, nc, (uint32_t)P.tasks.size(), 4, true).bytes);
+    if (state + 4 * 8 * (int64_t)P.sep_info.size() + 4096 > (int64_t)kStaticScratchBytes) return false;
+    const int32_t sep_levels = P.seg_lvl[np + 1] - 1 - P.seg_lvl[np];
+    if (33 * sep_levels <= nc - 730) return true;
+    std::vector<int64_t> terms(np + 1, 0);  // by the segment of their pivot
+    std::vector<int32_t> seg_of(nc, np);
+    for (int32_t q = 0; q < np; ++q)
+        for (int32_t p = P.seg_piv[q]; p < P.seg_piv[q + 1]; ++p) seg_of[p] = q;
+    for (const TermW& t : P.terms) ++terms[seg_of[t.m]];
+    const int64_t chain = *std::max_element(terms.begin(), terms.end() - 1) + terms[np];
+    // (the parts in all have about as many terms as one CTA's order: most molecules need no second plan)
+    if (4 * chain > (int64_t)P.terms.size()) return false;
+    one_cta.reset(new Program(choose_order(nc, na, adj, ci, cj, o, 1024)));  // kept if it is the one to use
+    return 4 * chain <= (int64_t)one_cta->terms.size();
+}
+
+// ------------------------------------------------------------------------------------
 // planning entry points (used by the C ABI in solve.cu)
 // ------------------------------------------------------------------------------------
 ilves_status plan_topology(ilves_topology* T, int32_t n_atoms, int32_t n_c, const int32_t* ai,
@@ -1131,12 +1228,7 @@ ilves_status plan_topology(ilves_topology* T, int32_t n_atoms, int32_t n_c, cons
         const int64_t wide_teams = (int64_t)kMaxSlotsPerCta * (T->n_sm > 0 ? T->n_sm : 152);
         if (n_batched > wide_teams && small * 10 >= batched * 9) narrow = kDefaultNarrowAtoms;
     }
-    // Automatic partition threshold: 4096 constraints, or kLonePartitionMin for a topology's only
-    // molecule that is too large for the batched kernel.  Its parts run on several SMs where one
-    // CTA has one SM's float64 pipe (a tree of 1400 atoms, mixed / float64: 119 / 242 us against
-    // 189 / 358; 4000 atoms: 154 / 326 against 425 / 767; even at 900 constraints).  Several such
-    // molecules share one launch of a CTA each, while partitioned solves run one after another.
-    constexpr int32_t kLonePartitionMin = 1000;
+    // molecules past the batched kernel's limits (see lone_partition_pays)
     int32_t n_big = 0;
     for (const MolHost& M : T->mols)
         if ((int32_t)M.cons.size() > warp_limit || (int32_t)M.cons.size() >= (int32_t)kCompactMaxConstraints ||
@@ -1207,50 +1299,21 @@ ilves_status plan_topology(ilves_topology* T, int32_t n_atoms, int32_t n_c, cons
             M.n_dom = 0;
             for (int32_t& v : M.dom_smem) v = 0;
         }
-        if (nc >= part_min || (o.partition_min_constraints <= 0 && n_big == 1 && M.large && nc >= kLonePartitionMin)) {
+        const bool lone = nc < part_min && o.partition_min_constraints <= 0 && n_big == 1 && M.large && nc >= kLonePartitionMin;
+        Program* parted = nc >= part_min || lone
+                              ? compile_parted(na, nc, adj, M.ci, M.cj, o, T->n_sm > 0 ? T->n_sm : 152,
+                                               lone ? kLoneMaxSeparators : nc)
+                              : nullptr;
+        std::unique_ptr<Program> one_cta;
+        if (parted && lone && !lone_partition_pays(*parted, na, nc, adj, M.ci, M.cj, o, one_cta)) {
+            delete parted;
+            parted = nullptr;
+        }
+        if (parted) {
             // partitioned: parts of ~part_size constraints eliminated first, separators last
+            Program* P = parted;
+            const int32_t np = P->n_seg - 1;
             M.large = M.parted = true;
-            // automatic part size: about 256 constraints, but never more parts (plus the
-            // separator CTA) than three CTAs per SM can keep resident, since the parts of a
-            // cooperative launch run at once with their programs in shared memory
-            int32_t part_size = o.part_constraints > 0 ? o.part_constraints : 256;
-            if (o.part_constraints <= 0) {
-                const int32_t max_parts = 3 * (T->n_sm > 0 ? T->n_sm : 152) - 1;
-                part_size = std::max(part_size, (nc + max_parts - 1) / max_parts);
-            }
-            const int32_t n_parts = std::max(2, std::min(8192, (nc + part_size - 1) / part_size));
-            std::vector<int32_t> bounds = partition_atoms(na, M.ci, M.cj, n_parts);
-            const int32_t np = (int32_t)bounds.size() - 1;
-            std::vector<int32_t> part_of(na);
-            for (int32_t q = 0; q < np; ++q)
-                for (int32_t a = bounds[q]; a < bounds[q + 1]; ++a) part_of[a] = q;
-            std::vector<int32_t> seg(nc);
-            std::vector<int8_t> stage(nc);
-            for (int32_t c = 0; c < nc; ++c) {
-                const bool inner = part_of[M.ci[c]] == part_of[M.cj[c]];
-                seg[c] = inner ? part_of[M.ci[c]] : np;
-                stage[c] = inner ? 0 : 1;
-            }
-            std::vector<int32_t> seg_atom(bounds);
-            seg_atom.push_back(na);  // the separator segment owns no atoms
-            // elimination order: rounds of independent pivots of near-minimum degree; the
-            // degree slack is tuned per molecule for the fewest levels in the deepest part
-            // (every level of a part costs a CTA barrier and a dependent chain, twice per
-            // iteration), then the fewest terms
-            Program* P = nullptr;
-            int64_t best_key = 0;
-            for (int32_t slack : {2, 3, 4, 6}) {
-                Program C = compile(nc, eliminate_rounds(nc, adj, slack, false, &stage), M.ci, M.cj, 256, na, &seg,
-                                    np + 1, &seg_atom);
-                int32_t deepest = 0;
-                for (int32_t q = 0; q < np; ++q) deepest = std::max(deepest, C.seg_lvl[q + 1] - 1 - C.seg_lvl[q]);
-                const int64_t key = ((int64_t)deepest << 40) + (int64_t)C.terms.size();
-                if (!P || key < best_key) {
-                    delete P;
-                    P = new Program(std::move(C));
-                    best_key = key;
-                }
-            }
             M.n_seg = np + 1;
             M.n_sept = (int32_t)P->sep_info.size();
             M.n_sep = nc - P->seg_piv[np];
@@ -1280,7 +1343,8 @@ ilves_status plan_topology(ilves_topology* T, int32_t n_atoms, int32_t n_c, cons
             continue;
         }
         M.team = (!M.large && na <= narrow) ? kNarrowThreads : kSlotThreads;
-        Program* P = new Program(choose_order(nc, na, adj, M.ci, M.cj, o, M.large ? 1024 : M.team));
+        Program* P = one_cta ? one_cta.release()
+                             : new Program(choose_order(nc, na, adj, M.ci, M.cj, o, M.large ? 1024 : M.team));
         if (!M.large && !fits_compact(*P)) {
             M.large = true;
             M.team = kSlotThreads;

@@ -16,8 +16,10 @@ A request carries one molecule topology (constrained atom pairs) and its coordin
   ordered, and each request completes on its own (its stream's event is polled), without
   waiting for the others.  A request's batched kernel launches only the CTAs that own its
   molecules (with the shared memory they use), so solves run side by side on disjoint SMs
-  rather than one after another; requests above the partition threshold are solved by
-  overlapping domains.  Each ilves_solve reads the request's page-locked host inputs and
+  rather than one after another; requests of 4096 constraints and more are solved by
+  overlapping domains, smaller ones past the batched kernel's limits by one CTA or, from 1000
+  constraints on and where the planner finds it faster, in parts with a Schur complement.
+  Each ilves_solve reads the request's page-locked host inputs and
   writes its page-locked host outputs in place (no staging copies) and computes the
   diagonal start itself,
 * records per-request latency (arrival -> results on the host), iterations and status;
