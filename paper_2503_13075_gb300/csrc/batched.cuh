@@ -302,7 +302,7 @@ struct BatchMol {
             }
             while (mine) {
                 const bool diag = HeadWord::diag(h);
-                const int s = (int)HeadWord::slot(h), np = (int)HeadWord::pairs(h);
+                const int s = (int)HeadWord::slot(h), nm = (int)HeadWord::more(h);
                 const uint2* tq = terms + HeadWord::first(h) + 1;  // the item's further term pairs
                 const V2 v = C[s];
                 LP e1, e2;  // float64: e1 alone, the sum of this lane
@@ -339,7 +339,7 @@ struct BatchMol {
                     term(xc.x);
                     term(xc.y);
 #pragma unroll 1
-                    for (int q = 1; q < np; ++q) {
+                    for (int q = 0; q < nm; ++q) {
                         const uint2 xn = x;
                         x = *++tq;
                         term(xn.x);

@@ -59,16 +59,17 @@ struct PairWord {
         return row | (col << 8) | ((atomsign >> 1) << 16) | ((atomsign & 1u) << 25);
     }
 };
-// HeadWord of an item that has terms: slot (12) | pivot (1) << 12 | pairs of terms (6) << 13 | its
-// first pair of terms (13) << 19.
+// HeadWord of an item that has terms: slot (12) | pivot (1) << 12 | pairs of terms past the first
+// (5) << 13 | its first pair of terms (14) << 18.  16384 pairs are 128 KB of terms; stars of
+// up to 57 bonds, whose factor is full, stay below (176 KB with their float64 values).
 struct HeadWord {
-    static constexpr uint32_t kMaxTerms = 63, kMaxPairs = 8192;
+    static constexpr uint32_t kMaxTerms = 63, kMaxPairs = 16384;
     static ILVES_HD uint32_t slot(uint32_t h) { return h & 0xFFFu; }
     static ILVES_HD bool diag(uint32_t h) { return ((h >> 12) & 1u) != 0u; }
-    static ILVES_HD uint32_t pairs(uint32_t h) { return (h >> 13) & 63u; }
-    static ILVES_HD uint32_t first(uint32_t h) { return h >> 19; }
+    static ILVES_HD uint32_t more(uint32_t h) { return (h >> 13) & 31u; }
+    static ILVES_HD uint32_t first(uint32_t h) { return h >> 18; }
     static ILVES_HD uint32_t make(uint32_t slot, bool diag, uint32_t pairs, uint32_t first) {
-        return slot | (diag ? 1u << 12 : 0u) | (pairs << 13) | (first << 19);
+        return slot | (diag ? 1u << 12 : 0u) | ((pairs - 1u) << 13) | (first << 18);
     }
 };
 // TermWord of item (j, q) and earlier pivot m: slots of the pairs (m, j) (12) and (m, q) (12) << 12
