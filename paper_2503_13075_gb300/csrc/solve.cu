@@ -2784,8 +2784,11 @@ extern "C" ilves_status ilves_autotune(ilves_topology* T, const double* x_old, c
     const float before = time_solves(T, x_old, x_unc, inv_mass, d, tol, precision, reps, s, buf, stat);
     if (before < 0.f) return ILVES_ERR_CUDA;
     // candidates: one knob at a time away from the current options
-    bool has_small = T->n_small > 0, has_parted = false;
-    for (const auto& M : T->mols) has_parted = has_parted || M.parted;
+    // (overlap depths only where a molecule reaches the threshold of overlapping domains: a lone
+    // molecule partitioned below it has the same plan at every depth)
+    bool has_small = T->n_small > 0, has_domains = false;
+    const int32_t domain_min = base.partition_min_constraints > 0 ? base.partition_min_constraints : 4096;
+    for (const auto& M : T->mols) has_domains = has_domains || (M.parted && (int32_t)M.cons.size() >= domain_min);
     std::vector<ilves_setup_opts> cands;
     auto add = [&](ilves_setup_opts c) {
         for (const auto& x : cands)
@@ -2815,7 +2818,7 @@ extern "C" ilves_status ilves_autotune(ilves_topology* T, const double* x_old, c
             add(c);
         }
     }
-    if (has_parted) {
+    if (has_domains) {
         for (int32_t ov : {0, 2, 3, 4, 6}) {
             ilves_setup_opts c = base;
             c.overlap = ov;
