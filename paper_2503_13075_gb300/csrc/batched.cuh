@@ -23,10 +23,12 @@
 //    teams and both kinds of solve have code of their own, so the passes' code has to stay in the
 //    instruction caches: unrolled four times by the compiler, 1.5 (float-float) and 0.6 (mixed)
 //    of a warp's stall cycles an issue were waits for instructions, 1.7 and 0.9 with one-warp teams
-//    beside the others; now 0.7 and 0.3 (135 -> 127 us mixed, 151 -> 129 us float-float).
+//    beside the others; now 0.7 and 0.3 (135 -> 127 us mixed, 151 -> 129 us float-float).  The copies
+//    of inputs and outputs are left to the compiler: rolled, every store of a multiplier waits for
+//    its index, which costs a batch on page-locked host buffers 5 % (4096 trees: 288 against 268 us).
 // Measured (4096 trees of 20-200 atoms, 96-thread teams; one task per entry and one atom per lane
-// before): mixed 162.0 -> 141.2 us, float64 541 -> 430 us; 8192 trees of 20-50 atoms on one-warp
-// teams 121.9 -> 100.1 us.  The mixed batch issues on two of five cycles (its teams wait on one
+// before): mixed 162.0 -> 132.4 us, float64 541 -> 417 us; 8192 trees of 20-50 atoms on one-warp
+// teams 121.7 -> 95.4 us.  The mixed batch issues on every other cycle (its teams wait on one
 // another and on shared memory); the float64 batch fills three quarters of the float64 pipe.
 #pragma once
 
@@ -39,9 +41,6 @@ struct BatchMol {
     struct alignas(2 * sizeof(LP)) V2 { LP x, y; };
     static constexpr bool DF = Mode::df;
     static constexpr bool kF32 = sizeof(LP) == 4;
-    // loops of copies: two at a time, except in the float-float mode, whose code is the largest
-    // (4096 chains of 64 atoms, mixed: 81.3 -> 79.8 us; 4096 trees, float-float: 128.9 against 131.8)
-    static constexpr int kCopies = DF ? 1 : 2;
     int na, nc, npair, nlevel, nover, zero;
     const BatchHead* head;
     const uint32_t* con;  // local atoms i | j << 16 of each position
@@ -116,20 +115,17 @@ struct BatchMol {
     //      start); inv_mass -> W, d -> D2, lambda0 -> LAM as raw values.  The reads run over atom
     //      slots, so consecutive lanes read consecutive addresses.
     __device__ __forceinline__ void s1_gather(int r0, int ts) {
-#pragma unroll 1
         for (int p = r0; p < nc; p += ts) {
             const int32_t g = gid_of_con(p);
             cp_async8(D2 + p, A.d + g);
             if (A.lambda0 && !A.start_diag) cp_async4(LAM + p, A.lambda0 + g);
         }
-#pragma unroll kCopies
         for (int e = r0; e < 3 * na; e += ts) {
             const int o = e / 3, c = e - 3 * o, a = (int)aslot[o];
             const int64_t g = 3 * slot_gid(o) + c;
             cp_async8(STG + 3 * a + c, A.x_old + g);
             cp_async8(DF ? X + 3 * a + c : X + c * na + a, A.x_unc + g);
         }
-#pragma unroll kCopies
         for (int o = r0; o < na; o += ts) cp_async8(W + aslot[o], A.inv_mass + slot_gid(o));
         cp_async_wait_all();
     }
@@ -562,7 +558,6 @@ struct BatchMol {
 
     // ---- S7: the positions, one coordinate per lane in global order; the multipliers
     __device__ __forceinline__ void out_atoms(int r0, int ts) {
-#pragma unroll kCopies
         for (int e = r0; e < 3 * na; e += ts) {
             const int o = e / 3, c = e - 3 * o, a = (int)aslot[o];
             const int64_t g = 3 * slot_gid(o) + c;
@@ -642,7 +637,6 @@ __device__ void solve_batched(const Team& tm, const MolDesc& D, const BatchLayou
     }
     M.out_atoms(r0, ts);
     if (A.lambda_out)
-#pragma unroll 1
         for (int p = r0; p < nc; p += ts) M.out_lambda(p);
     if (r0 == 0) {
         if (A.iterations_out) A.iterations_out[D.mol_id] = iters;
