@@ -556,12 +556,20 @@ struct BatchMol {
         return reinterpret_cast<const double*>(kF32 ? (const void*)RF : (const void*)&PV[0].y);
     }
 
-    // ---- S7: the positions, one coordinate per lane in global order; the multipliers
+    // ---- S7: the positions, one coordinate per lane in global order; the multipliers.  The
+    //      float-float mode adds x_unc, which it reads again: first, all of a lane's coordinates at
+    //      once (into the rows' space, free by now), since a read behind each write is a
+    //      round trip each, over the host link a long one (x_out may be x_unc): 2500 trees on
+    //      page-locked buffers 238 -> 210 us.
     __device__ __forceinline__ void out_atoms(int r0, int ts) {
+        if constexpr (DF) {
+            for (int e = r0; e < 3 * na; e += ts) cp_async8(STG + e, A.x_unc + 3 * slot_gid(e / 3) + e % 3);
+            cp_async_wait_all();
+        }
         for (int e = r0; e < 3 * na; e += ts) {
             const int o = e / 3, c = e - 3 * o, a = (int)aslot[o];
             const int64_t g = 3 * slot_gid(o) + c;
-            if constexpr (DF) A.x_out[g] = A.x_unc[g] + df_join(as_df(X[c * na + a]));
+            if constexpr (DF) A.x_out[g] = STG[e] + df_join(as_df(X[c * na + a]));
             else A.x_out[g] = X[c * na + a];
         }
     }
