@@ -38,13 +38,14 @@ constexpr uint32_t kNoAtom32 = 0xFFFFFFFFu;
 //         (sign product < 0), the dummy atom for fill entries, unused for DIAG tasks;
 //         tstart = first term.  Task t's terms are [tstart_t, tstart_{t+1}); a sentinel
 //         task ends the list.
-//   Term: l = slot of Lt[row, m], u = slot of U[m, col], m = the earlier pivot.
+//   TermWide: l = slot of Lt[row, m], u = slot of U[m, col], m = the earlier pivot.
 //   Piv:  diag = first slot of the pivot's U row (its L column follows), nup = |N+(pivot)|.
 //   ConA: local atom ids (i, j) of the constraint at position p.
 // inc[e] = p << 1 | (atom is the second atom of constraint p)
-template <class IdxT> struct Task { IdxT row, col, atomsign, tstart; };
-template <class IdxT> struct ConA { IdxT i, j; };
-template <class IdxT> struct Piv { IdxT diag, nup; };
+struct Task { uint32_t row, col, atomsign, tstart; };
+struct ConA { uint32_t i, j; };
+struct Piv { uint32_t diag, nup; };
+struct TermWide { uint32_t l, u, m, pad; };
 
 // Words of a batched molecule's program.  Its values are two to a slot: off-diagonal pair k of the
 // factor (U[j,q], L[q,j]), then pivot p at batch_pivot_base + p, then a zero.
@@ -91,17 +92,6 @@ struct BackWord {
 #endif
 constexpr uint32_t kNoInc = 0x8000u;  // an absent incidence of a batched molecule's atom
 
-// Term words of large molecules: 4 x 32 bits.
-struct TermWide { uint32_t l, u, m, pad; };
-template <class IdxT> struct TermOf;
-template <> struct TermOf<uint32_t> {
-    using T = TermWide;
-    using TaskT = Task<uint32_t>;
-    static ILVES_HD uint32_t l(T t) { return t.l; }
-    static ILVES_HD uint32_t u(T t) { return t.u; }
-    static ILVES_HD uint32_t m(T t) { return t.m; }
-    static ILVES_HD T make(uint32_t l, uint32_t u, uint32_t m) { return TermWide{l, u, m, 0u}; }
-};
 constexpr uint32_t kCompactMaxConstraints = 256, kCompactMaxSlots = 4096;
 // Threads of the team that solves one molecule of the batched kernel (whole warps; three
 // warps cut the passes of wide levels at no cost in residency, which shared memory
@@ -379,22 +369,20 @@ ILVES_HD DomStateLayout dom_state_layout(uint32_t na, uint32_t na_own, uint32_t 
 // separators (constraints between parts), whose atom range is empty.
 struct SegRow { int32_t piv, lvl, atom; };
 
-template <class IdxT>
 ILVES_HD ProgLayout prog_layout(uint32_t na, uint32_t nc, uint32_t ntask, uint32_t nterm,
                                 uint32_t nlevel, uint32_t n_seg = 1, uint32_t n_sept = 0, uint32_t n_cent = 0,
                                 uint32_t pprog_bytes = 0) {
     ProgLayout L;
-    const uint32_t ix = (uint32_t)sizeof(IdxT);
     uint32_t o = 0;
     L.seg = o;       o = align16(o + 12u * (n_seg + 1));
-    L.con_atoms = o; o = align16(o + 2u * ix * nc);
-    L.piv = o;       o = align16(o + 2u * ix * nc);
-    L.lvl_task = o;  o = align16(o + ix * (nlevel + 1));
-    L.lvl_piv = o;   o = align16(o + ix * (nlevel + 1));
-    L.inc_ptr = o;   o = align16(o + ix * (na + 1));
-    L.inc = o;       o = align16(o + ix * 2u * nc);
-    L.tasks = o;     o = align16(o + 4u * ix * (ntask + 1));
-    L.terms = o;     o = align16(o + (uint32_t)sizeof(typename TermOf<IdxT>::T) * nterm);
+    L.con_atoms = o; o = align16(o + (uint32_t)sizeof(ConA) * nc);
+    L.piv = o;       o = align16(o + (uint32_t)sizeof(Piv) * nc);
+    L.lvl_task = o;  o = align16(o + 4u * (nlevel + 1));
+    L.lvl_piv = o;   o = align16(o + 4u * (nlevel + 1));
+    L.inc_ptr = o;   o = align16(o + 4u * (na + 1));
+    L.inc = o;       o = align16(o + 8u * nc);
+    L.tasks = o;     o = align16(o + (uint32_t)sizeof(Task) * (ntask + 1));
+    L.terms = o;     o = align16(o + (uint32_t)sizeof(TermWide) * nterm);
     const bool parted = n_seg > 1;
     L.sep_info = o;  o = align16(o + (parted ? 8u * n_sept : 0u));
     L.cptr = o;      o = align16(o + (parted ? 4u * n_seg : 0u));  // n_parts + 1 = n_seg entries

@@ -296,24 +296,22 @@ __device__ __forceinline__ T ldp(const T* p) {
     }
 }
 
-template <class Mode, class IdxT, bool kCoh>
+template <class Mode, bool kCoh>
 struct MolView {
     using LP = typename Mode::LP;
     using V4 = typename Mode::V4;
-    using TO = TermOf<IdxT>;
-    using TaskT = typename TO::TaskT;
     static constexpr bool DF = Mode::df;
     int na, nc;
     const SegRow* seg;
-    const ConA<IdxT>* con;
+    const ConA* con;
     const int32_t* con_gid;
-    const Piv<IdxT>* piv;
-    const IdxT* lvl_task;
-    const IdxT* lvl_piv;
-    const IdxT* inc_ptr;
-    const IdxT* inc;
-    const TaskT* tasks;
-    const typename TO::T* terms;
+    const Piv* piv;
+    const uint32_t* lvl_task;
+    const uint32_t* lvl_piv;
+    const uint32_t* inc_ptr;
+    const uint32_t* inc;
+    const Task* tasks;
+    const TermWide* terms;
     double *X, *W, *RHO, *SK, *D2, *LAM;
     float* RHOL;  // float-float mode: low parts of rho (SoA); the high parts are RHOF.xyz
     LP *WL, *Y, *V;
@@ -341,18 +339,18 @@ struct MolView {
         na = d.na;
         nc = d.nc;
         const ProgLayout PL =
-            prog_layout<IdxT>(na, nc, d.ntask, d.nterm, d.nlevel, d.n_seg, d.n_sept, d.n_cent, d.pprog_bytes);
+            prog_layout(na, nc, d.ntask, d.nterm, d.nlevel, d.n_seg, d.n_sept, d.n_cent, d.pprog_bytes);
         const StateLayout SL = state_layout(na, nc, d.ntask, sizeof(LP), DF);
         seg = reinterpret_cast<const SegRow*>(prog + PL.seg);
-        con = reinterpret_cast<const ConA<IdxT>*>(prog + PL.con_atoms);
+        con = reinterpret_cast<const ConA*>(prog + PL.con_atoms);
         con_gid = reinterpret_cast<const int32_t*>(gprog + PL.con_gid);
-        piv = reinterpret_cast<const Piv<IdxT>*>(prog + PL.piv);
-        lvl_task = reinterpret_cast<const IdxT*>(prog + PL.lvl_task);
-        lvl_piv = reinterpret_cast<const IdxT*>(prog + PL.lvl_piv);
-        inc_ptr = reinterpret_cast<const IdxT*>(prog + PL.inc_ptr);
-        inc = reinterpret_cast<const IdxT*>(prog + PL.inc);
-        tasks = reinterpret_cast<const TaskT*>(prog + PL.tasks);
-        terms = reinterpret_cast<const typename TO::T*>(prog + PL.terms);
+        piv = reinterpret_cast<const Piv*>(prog + PL.piv);
+        lvl_task = reinterpret_cast<const uint32_t*>(prog + PL.lvl_task);
+        lvl_piv = reinterpret_cast<const uint32_t*>(prog + PL.lvl_piv);
+        inc_ptr = reinterpret_cast<const uint32_t*>(prog + PL.inc_ptr);
+        inc = reinterpret_cast<const uint32_t*>(prog + PL.inc);
+        tasks = reinterpret_cast<const Task*>(prog + PL.tasks);
+        terms = reinterpret_cast<const TermWide*>(prog + PL.terms);
         X = reinterpret_cast<double*>(st + SL.x);
         W = reinterpret_cast<double*>(st + SL.w);
         WL = reinterpret_cast<LP*>(st + SL.wl);
@@ -377,7 +375,7 @@ struct MolView {
     __device__ __forceinline__ int64_t gid(int a) const {
         return D->atom_base >= 0 ? (int64_t)D->atom_base + a : (int64_t)A->atom_gid[D->gid_off + a];
     }
-    __device__ __forceinline__ ConA<IdxT> cons(int p) const { return ldp<kCoh>(con + p); }
+    __device__ __forceinline__ ConA cons(int p) const { return ldp<kCoh>(con + p); }
     __device__ __forceinline__ int32_t gid_of_con(int p) const { return __ldg(con_gid + p); }
     __device__ __forceinline__ LP* inv_ptr(int p) const { return reinterpret_cast<LP*>(RF + p) + 3; }
     __device__ __forceinline__ bool foreign(int p) const { return cohall || p >= sep_p0; }
@@ -603,7 +601,7 @@ struct MolView {
     // global); part_staged (partitioned, both atoms in the CTA's part): x_old in X, x_unc
     // in the part copy XS, weights in WL, so the inputs are read once per atom, in order
     __device__ __forceinline__ void s1_constraint(int p, bool ref_staged, bool part_staged = false) {
-        const ConA<IdxT> c = cons(p);
+        const ConA c = cons(p);
         const int i = c.i, j = c.j;
         const int64_t gi = gid(i), gj = gid(j);
         ref_staged = ref_staged || part_staged;
@@ -729,7 +727,7 @@ struct MolView {
     //      Jacobian rows are not needed).
     struct Viol { V4 v; LP y; bool conv, bad; };
     __device__ __forceinline__ Viol viol_eval(int p) const {
-        const ConA<IdxT> cc = cons(p);
+        const ConA cc = cons(p);
         const int i = cc.i, j = cc.j;
         const bool fx = foreign(p);
         Viol o;
@@ -807,10 +805,10 @@ struct MolView {
 #pragma unroll 2
         for (int e = e0; e < e1; ++e) {
             const auto tr = ldp<kCoh>(terms + e);
-            const int m = TO::m(tr);
+            const int m = tr.m;
             const bool fm = foreign(m);
-            const LP li = v_ld(TO::l(tr), fm) * inv(m);
-            sacc -= li * v_ld(TO::u(tr), fm);
+            const LP li = v_ld(tr.l, fm) * inv(m);
+            sacc -= li * v_ld(tr.u, fm);
             if (diag) yv += li * y_ld(m);
         }
         v_st(t, sacc);
@@ -822,7 +820,7 @@ struct MolView {
     }
     // large molecules: task records with term pointers
     __device__ __forceinline__ void task(int t, bool diag, bool& singular) {
-        const TaskT tk = ldp<kCoh>(tasks + t);
+        const Task tk = ldp<kCoh>(tasks + t);
         const int e1 = ldp<kCoh>(tasks + t + 1).tstart;
         task_core(t, tk.row, tk.col, tk.atomsign >> 1, tk.atomsign & 1, tk.tstart, e1, diag, singular);
     }
@@ -832,9 +830,9 @@ struct MolView {
         LP yv = LP(0);
         for (int e = e0; e < e1; ++e) {
             const auto tr = ldp<kCoh>(terms + e);
-            const int m = TO::m(tr);
+            const int m = tr.m;
             const bool fm = foreign(m);
-            yv += v_ld(TO::l(tr), fm) * inv(m) * y_ld(m);
+            yv += v_ld(tr.l, fm) * inv(m) * y_ld(m);
         }
         y_st(p, y_ld(p) - yv);
     }
@@ -847,7 +845,7 @@ struct MolView {
     // ---- backward S5 for pivot p: delta_p = inv_p (y_p - sum_q U[p,q] delta_q)
     __device__ __forceinline__ int task_col(int t) const { return (int)ldp<kCoh>(tasks + t).col; }
     __device__ __forceinline__ void backward(int p) {
-        const Piv<IdxT> pv = ldp<kCoh>(piv + p);
+        const Piv pv = ldp<kCoh>(piv + p);
         const int us = pv.diag, nu = pv.nup;
         const bool fp = foreign(p);
         LP dl = y_ld(p);
@@ -861,15 +859,15 @@ struct MolView {
     //      sum as well; DIAG tasks: the L inv y sum of the forward solve)
     __device__ __forceinline__ void contrib(int c, bool factor) {
         const Contrib E = ldp<kCoh>(cent + c);
-        const TaskT tk = ldp<kCoh>(tasks + E.task);
+        const Task tk = ldp<kCoh>(tasks + E.task);
         const bool diag = tk.row == tk.col;
         LP sv = LP(0), sy = LP(0);
         for (uint32_t e = E.e0; e < E.e1; ++e) {
             const auto tr = ldp<kCoh>(terms + e);
-            const int m = TO::m(tr);
+            const int m = tr.m;
             const bool fm = foreign(m);
-            const LP li = v_ld(TO::l(tr), fm) * inv(m);
-            if (factor) sv += li * v_ld(TO::u(tr), fm);
+            const LP li = v_ld(tr.l, fm) * inv(m);
+            if (factor) sv += li * v_ld(tr.u, fm);
             if (diag) sy += li * y_ld(m);
         }
         LP* ct = CT + 4 * (E.task - sep_t0);
@@ -878,7 +876,7 @@ struct MolView {
     }
     // separator task t: the parts' contributions, then its remaining terms
     __device__ __forceinline__ void task_sep(int t, bool diag, bool& singular) {
-        const TaskT tk = ldp<kCoh>(tasks + t);
+        const Task tk = ldp<kCoh>(tasks + t);
         const int e1 = ldp<kCoh>(tasks + t + 1).tstart;
         const SepInfo si = ldp<kCoh>(sep_info + (t - sep_t0));
         const LP a = assemble(tk.row, tk.col, tk.atomsign >> 1, tk.atomsign & 1, diag);
@@ -890,9 +888,9 @@ struct MolView {
         }
         for (int e = (int)si.b_start; e < e1; ++e) {
             const auto tr = ldp<kCoh>(terms + e);
-            const int m = TO::m(tr);
-            const LP li = lds<kCoh>(V + TO::l(tr)) * inv(m);
-            sacc -= li * lds<kCoh>(V + TO::u(tr));
+            const int m = tr.m;
+            const LP li = lds<kCoh>(V + tr.l) * inv(m);
+            sacc -= li * lds<kCoh>(V + tr.u);
             if (diag) yv += li * lds<kCoh>(Y + m);
         }
         V[t] = sacc;
@@ -911,8 +909,8 @@ struct MolView {
         const int e1 = ldp<kCoh>(tasks + t + 1).tstart;
         for (int e = (int)si.b_start; e < e1; ++e) {
             const auto tr = ldp<kCoh>(terms + e);
-            const int m = TO::m(tr);
-            yv += lds<kCoh>(V + TO::l(tr)) * inv(m) * lds<kCoh>(Y + m);
+            const int m = tr.m;
+            yv += lds<kCoh>(V + tr.l) * inv(m) * lds<kCoh>(Y + m);
         }
         Y[p] = lds<kCoh>(Y + p) - yv;
     }
@@ -946,9 +944,9 @@ struct MolView {
             ym = SY[m];
         } else {  // an interior pivot past the parts' two contribution slots
             const auto g = ldp<kCoh>(terms + tr.y);
-            const int m = TO::m(g);
-            li = lds<kCoh>(V + TO::l(g)) * lds<kCoh>(inv_ptr(m));
-            u = lds<kCoh>(V + TO::u(g));
+            const int m = g.m;
+            li = lds<kCoh>(V + g.l) * lds<kCoh>(inv_ptr(m));
+            u = lds<kCoh>(V + g.u);
             ym = lds<kCoh>(Y + m);
         }
     }
@@ -1048,7 +1046,7 @@ struct MolView {
     }
     // assembly coefficient 4 s s' w of separator task tl (w_i + w_j for a pivot)
     __device__ __forceinline__ LP sep_coef(int tl) const {
-        const TaskT tk = ldp<kCoh>(tasks + sep_t0 + tl);
+        const Task tk = ldp<kCoh>(tasks + sep_t0 + tl);
         const LP wv = tk.row == tk.col ? lds<kCoh>(RHOF + tk.row).w : lds<kCoh>(WL + (tk.atomsign >> 1));
         return (tk.atomsign & 1) ? LP(-4) * wv : LP(4) * wv;
     }
@@ -1091,7 +1089,7 @@ struct MolView {
 template <class Mode>
 __device__ void solve_molecule(const BlockTeam& tm, const MolDesc& D, const uint8_t* prog, uint8_t* st,
                                const SolveArgs& A) {
-    MolView<Mode, uint32_t, false> M;
+    MolView<Mode, false> M;
     M.init(D, prog, st, A, prog);
     const int na = D.na, nc = D.nc;
     const int r0 = tm.rank(), ts = tm.size();
@@ -1274,7 +1272,7 @@ k_solve_parted(const MolDesc* __restrict__ desc, const uint8_t* __restrict__ blo
     using V4 = typename Mode::V4;
     extern __shared__ __align__(16) uint8_t sep_smem[];
     const MolDesc D = *desc;
-    MolView<Mode, uint32_t, true> M;
+    MolView<Mode, true> M;
     M.init(D, blob + D.blob_off, work + D.work_off, A, blob + D.blob_off);
     const int n_parts = D.n_seg - 1;
     const SegRow* seg = M.seg;
@@ -1292,7 +1290,7 @@ k_solve_parted(const MolDesc* __restrict__ desc, const uint8_t* __restrict__ blo
         reinterpret_cast<uint8_t*>(CS) + (cfg.sep_ct ? align16(4u * (uint32_t)sizeof(LP) * D.n_sept) : 0u);
     // segment programs: part q's is [poff[q], poff[q + 1]) of the pprog section, the
     // separator block's follows
-    const ProgLayout PL = prog_layout<uint32_t>(D.na, D.nc, D.ntask, D.nterm, D.nlevel, D.n_seg, D.n_sept, D.n_cent,
+    const ProgLayout PL = prog_layout(D.na, D.nc, D.ntask, D.nterm, D.nlevel, D.n_seg, D.n_sept, D.n_cent,
                                                 D.pprog_bytes);
     const uint8_t* gp = blob + D.blob_off;
     const uint32_t* poff = reinterpret_cast<const uint32_t*>(gp + PL.pprog_off);

@@ -806,37 +806,36 @@ static Program choose_order(int32_t nc, int32_t na, const std::vector<std::vecto
 // blob writers (large molecules, batched molecules)
 // ------------------------------------------------------------------------------------
 static ProgLayout layout_for(const MolHost& M) {
-    return prog_layout<uint32_t>((uint32_t)M.atoms.size(), (uint32_t)M.cons.size(), (uint32_t)M.ntask,
+    return prog_layout((uint32_t)M.atoms.size(), (uint32_t)M.cons.size(), (uint32_t)M.ntask,
                              (uint32_t)M.nterm, (uint32_t)M.nlevel, (uint32_t)M.n_seg, (uint32_t)M.n_sept,
                              (uint32_t)M.n_cent, (uint32_t)M.pprog_bytes);
 }
 
 static void write_blob(uint8_t* dst, const MolHost& M, const Program& P) {
-    using IdxT = uint32_t;
     const ProgLayout L = layout_for(M);
     std::memset(dst, 0, L.bytes);
     auto* seg = reinterpret_cast<SegRow*>(dst + L.seg);
     for (int32_t g = 0; g <= P.n_seg; ++g) seg[g] = SegRow{P.seg_piv[g], P.seg_lvl[g], P.seg_atom[g]};
-    auto* con = reinterpret_cast<ConA<IdxT>*>(dst + L.con_atoms);
+    auto* con = reinterpret_cast<ConA*>(dst + L.con_atoms);
     auto* con_gid = reinterpret_cast<int32_t*>(dst + L.con_gid);
-    auto* piv = reinterpret_cast<Piv<IdxT>*>(dst + L.piv);
-    auto* lvl_task = reinterpret_cast<IdxT*>(dst + L.lvl_task);
-    auto* lvl_piv = reinterpret_cast<IdxT*>(dst + L.lvl_piv);
-    auto* inc_ptr = reinterpret_cast<IdxT*>(dst + L.inc_ptr);
-    auto* inc = reinterpret_cast<IdxT*>(dst + L.inc);
-    auto* terms = reinterpret_cast<typename TermOf<IdxT>::T*>(dst + L.terms);
+    auto* piv = reinterpret_cast<Piv*>(dst + L.piv);
+    auto* lvl_task = reinterpret_cast<uint32_t*>(dst + L.lvl_task);
+    auto* lvl_piv = reinterpret_cast<uint32_t*>(dst + L.lvl_piv);
+    auto* inc_ptr = reinterpret_cast<uint32_t*>(dst + L.inc_ptr);
+    auto* inc = reinterpret_cast<uint32_t*>(dst + L.inc);
+    auto* terms = reinterpret_cast<TermWide*>(dst + L.terms);
     const int32_t nc = (int32_t)M.cons.size(), na = (int32_t)M.atoms.size();
     for (int32_t p = 0; p < nc; ++p) {
         const int32_t c = P.pos_con[p];
-        con[p].i = (IdxT)M.ci[c];
-        con[p].j = (IdxT)M.cj[c];
+        con[p].i = (uint32_t)M.ci[c];
+        con[p].j = (uint32_t)M.cj[c];
         con_gid[p] = M.cons[c];
-        piv[p].diag = (IdxT)P.ustart[p];
-        piv[p].nup = (IdxT)P.up[p].size();
+        piv[p].diag = (uint32_t)P.ustart[p];
+        piv[p].nup = (uint32_t)P.up[p].size();
     }
     for (size_t l = 0; l < P.lvl_piv.size(); ++l) {
-        lvl_task[l] = (IdxT)P.lvl_task[l];
-        lvl_piv[l] = (IdxT)P.lvl_piv[l];
+        lvl_task[l] = (uint32_t)P.lvl_task[l];
+        lvl_piv[l] = (uint32_t)P.lvl_piv[l];
     }
     std::vector<int32_t> cnt(na + 1, 0);
     for (int32_t p = 0; p < nc; ++p) {
@@ -844,23 +843,16 @@ static void write_blob(uint8_t* dst, const MolHost& M, const Program& P) {
         ++cnt[con[p].j + 1];
     }
     for (int32_t a = 0; a < na; ++a) cnt[a + 1] += cnt[a];
-    for (int32_t a = 0; a <= na; ++a) inc_ptr[a] = (IdxT)cnt[a];
+    for (int32_t a = 0; a <= na; ++a) inc_ptr[a] = (uint32_t)cnt[a];
     std::vector<int32_t> fillp(cnt.begin(), cnt.end() - 1);
     for (int32_t p = 0; p < nc; ++p) {
-        inc[fillp[con[p].i]++] = (IdxT)((uint32_t)p << 1);
-        inc[fillp[con[p].j]++] = (IdxT)(((uint32_t)p << 1) | 1u);
+        inc[fillp[con[p].i]++] = (uint32_t)p << 1;
+        inc[fillp[con[p].j]++] = ((uint32_t)p << 1) | 1u;
     }
-    auto term_of = [&](size_t k) { return TermOf<IdxT>::make(P.terms[k].l, P.terms[k].u, P.terms[k].m); };
-    auto* tasks = reinterpret_cast<Task<IdxT>*>(dst + L.tasks);
-    const IdxT no_atom = (IdxT)~(IdxT)0;
-    for (size_t t = 0; t < P.tasks.size(); ++t) {
-        const TaskW& w = P.tasks[t];
-        tasks[t].row = (IdxT)w.row;
-        tasks[t].col = (IdxT)w.col;
-        tasks[t].atomsign = w.atomsign == kNoAtom32 ? no_atom : (IdxT)w.atomsign;  // sentinel
-        tasks[t].tstart = (IdxT)w.tstart;
-    }
-    for (size_t k = 0; k < P.terms.size(); ++k) terms[k] = term_of(k);
+    auto* tasks = reinterpret_cast<Task*>(dst + L.tasks);
+    for (size_t t = 0; t < P.tasks.size(); ++t)
+        tasks[t] = Task{P.tasks[t].row, P.tasks[t].col, P.tasks[t].atomsign, P.tasks[t].tstart};
+    for (size_t k = 0; k < P.terms.size(); ++k) terms[k] = TermWide{P.terms[k].l, P.terms[k].u, P.terms[k].m, 0u};
     if (P.n_seg > 1) {
         std::memcpy(dst + L.sep_info, P.sep_info.data(), P.sep_info.size() * sizeof(SepInfo));
         std::memcpy(dst + L.cptr, P.cptr.data(), P.cptr.size() * sizeof(int32_t));
