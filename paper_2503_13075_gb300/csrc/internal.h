@@ -107,9 +107,10 @@ constexpr int kMaxSlotsPerCta = kSlotCtaThreads / kSlotThreads;
 // Narrow class: molecules of at most narrow_atoms atoms get one-warp teams, up to
 // kNarrowSlotsPerCta per CTA beside its 96-thread teams.  Their slices are small, so an SM's
 // shared memory holds about three times as many of them: a batch of 4096 trees of 50-100 atoms
-// (mixed) takes 96 us against 117 on 96-thread teams.  On batches of mixed sizes (20-200
-// atoms) they lose (145 us and more against 141), so the automatic choice keeps those on 96
-// threads and leaves the threshold to the autotuner.
+// (mixed) takes 87 us against 108 on 96-thread teams, 8192 of 20-50 atoms 95 against 141.  On
+// batches of mixed sizes (20-200 atoms, mixed / float64 / float-float) they gain 3 % at best and
+// lose in the other precisions (up to 60 atoms: 124 / 344 / 143 us against 127 / 327 / 131), so
+// the automatic choice keeps those on 96 threads and leaves the threshold to the autotuner.
 constexpr int kNarrowThreads = 32;
 constexpr int kNarrowSlotsPerCta = kSlotCtaThreads / kNarrowThreads;
 constexpr int kDefaultNarrowAtoms = 100;

@@ -277,7 +277,7 @@ static_assert(4 * (SM_REQUEST + 1024) > 228 * 1024 && kTmemCols * 3 <= 512, "at 
 // gathers (two dependent rounds, about 3,700 cycles with three CTAs to an SM) and the two
 // epilogues' 128 columns a row (about 2,200 each).  Two threads to a row halve both chains and
 // double the warps an SM overlaps them with (24 on three CTAs): a warm start of 258,048
-// constraints, with its prep pass, 50.6 -> 43.7 us.
+// constraints, with its prep pass, 50.6 -> 43.7 us, and 37.7 as a dependent launch.
 template <bool kFused, bool kTrain>
 __global__ void __launch_bounds__(kFwdThreads, 3)
 k_mlp_forward(MlpWeights Wt, const float* __restrict__ X, int n, FeatArgs F, float* __restrict__ out,
@@ -477,8 +477,9 @@ k_mlp_forward(MlpWeights Wt, const float* __restrict__ X, int n, FeatArgs F, flo
 // the gradient is the same on every run and its rounding error does not grow with the number
 // of CTAs, as it did with float32 atomics.  Rows are spread over the SMs, but at least kBwdMinRows
 // to a CTA, below which the 75 KB of W2 in and gradient out cost more than they save.
-// A whole gradient of 8192 rows takes 38.9 us (forward 12, this kernel 20, reduction 5); with one thread per hidden unit, rows streamed one by
-// one with three barriers each and float32 atomics it took 220 us.
+// A whole gradient of 8192 rows takes 32.8 us (38.9 before its kernels were dependent launches:
+// forward 12, this kernel 20, reduction 5); with one thread per hidden unit, rows streamed one
+// by one with three barriers each and float32 atomics it took 227 us.
 constexpr int kBwdRows = 64, kBwdMinRows = 16, kBwdThreads = 256;
 constexpr int kPartStride = (P_N + 1 + 3) & ~3;  // a CTA's partial gradient, then its loss
 constexpr int kBwdSmem = (NH * NH + 2 * kBwdRows * NH + kBwdRows * NF + kBwdRows) * (int)sizeof(float);

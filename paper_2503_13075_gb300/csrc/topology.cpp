@@ -1204,9 +1204,9 @@ ilves_status plan_topology(ilves_topology* T, int32_t n_atoms, int32_t n_c, cons
     // most that many atoms.  Default (0): kDefaultNarrowAtoms, but only for a batch made of
     // such molecules -- at least 90 % of the batched atoms, and more batched molecules than
     // the wide teams the GPU holds (eight per SM) -- where one-warp teams measured faster (50-100
-    // atoms: 96 us against 117); on batches of mixed sizes they are slower in every precision
-    // (20-200 atoms, one-warp teams up to 60: mixed 145 us against 141, float64 508 against 469,
-    // float-float 164 against 152); a lone molecule finishes sooner on 96 threads.
+    // atoms: 87 us against 108); on batches of mixed sizes it depends on the precision (20-200
+    // atoms, one-warp teams up to 60: mixed 124 us against 127, float64 344 against 327,
+    // float-float 143 against 131); a lone molecule finishes sooner on 96 threads.
     int32_t narrow = o.narrow_atoms > 0 ? o.narrow_atoms : -1;
     if (o.narrow_atoms == 0) {
         int64_t batched = 0, small = 0, n_batched = 0;
